@@ -204,11 +204,12 @@ struct Model {
     float *ftab32 = nullptr;
     FusedTables<double> f64() const
     {
-        return {ftab64, ftab64 + tab_n, ftab64 + 2 * tab_n, ftab64 + 3 * tab_n, ftab64 + 3 * tab_n + 2 * np};
+        return {ftab64, ftab64 + tab_n, ftab64 + 2 * tab_n, ftab64 + 3 * tab_n, ftab64 + 3 * tab_n + 2 * np,
+                reinterpret_cast<const int *>(ftab64 + 3 * tab_n + 3 * np)};
     }
     FusedTables<float> f32() const
     {
-        return {ftab32, ftab32 + tab_n, ftab32 + 2 * tab_n, ftab32 + 3 * tab_n, ftab32 + 3 * tab_n + 2 * np};
+        return {ftab32, ftab32 + tab_n, ftab32 + 2 * tab_n, ftab32 + 3 * tab_n, ftab32 + 3 * tab_n + 2 * np, nullptr};
     }
     ~Model()
     {
@@ -560,9 +561,31 @@ qhfpe_status build_model(qhfpe *h, Model &M, int S, const double *U, const doubl
     if (M.fused) {
         std::vector<double> ft;
         build_tables(M, U, ft, [&](int pos) { return fused_fft_frequency(p.np, pos); }, p.np, true);
+        std::vector<float> ft32(ft.begin(), ft.end());
+        // the FP64 form's transforms and mixing run on integers (FusedTables): twiddles times 2^62, each row of a
+        // table times 2^(62 - k) with 2^k above its largest value; the exponents k follow
+        for (int t = 0; t < 2 * p.np; ++t) {
+            const long double a = 2.0L * std::acos(-1.0L) * (t / 2) / p.np;
+            const long long w = std::llrint((t % 2 ? std::sin(a) : std::cos(a)) * 0x1p62L);
+            std::memcpy(&ft[3 * M.tab_n + t], &w, sizeof(w));
+        }
+        const size_t n_rows = 3 * M.tab_n / p.np;
+        std::vector<int> kx(n_rows + n_rows % 2, 0);
+        for (size_t r = 0; r < n_rows; ++r) {
+            double *row = ft.data() + r * p.np, big = 0.0;
+            for (int t = 0; t < p.np; ++t) big = std::max(big, std::fabs(row[t]));
+            int k = -4096;  // a row of zeros: below every other term
+            if (big > 0.0) std::frexp(big, &k);
+            kx[r] = k;
+            for (int t = 0; t < p.np; ++t) {
+                const long long c = big > 0.0 ? std::llrint(std::ldexp(row[t], 62 - k)) : 0;
+                std::memcpy(row + t, &c, sizeof(c));
+            }
+        }
+        ft.resize(3 * M.tab_n + 3 * p.np + kx.size() / 2);
+        std::memcpy(ft.data() + 3 * M.tab_n + 3 * p.np, kx.data(), kx.size() * sizeof(int));
         QH_CK(h, dalloc(&M.ftab64, ft.size()));
         QH_CK(h, cudaMemcpyAsync(M.ftab64, ft.data(), sizeof(double) * ft.size(), cudaMemcpyHostToDevice, st));
-        std::vector<float> ft32(ft.begin(), ft.end());
         QH_CK(h, dalloc(&M.ftab32, ft32.size()));
         QH_CK(h, cudaMemcpyAsync(M.ftab32, ft32.data(), sizeof(float) * ft32.size(), cudaMemcpyHostToDevice, st));
         QH_CK(h, (prepare_fused<float, true>(p.np, S)));

@@ -33,7 +33,12 @@ dipole_fft_kernel(GridInfo g, const T *__restrict__ TL, const T *__restrict__ TR
     const int i0 = tile * tq, rows = min(tq, nq - i0);
     const size_t blk = g.blk;
     T *base = state + (size_t)rep * rep_stride + (size_t)e * g.elem_stride;
-    for (int t = threadIdx.x; t < NP; t += FTHREADS) tw[t] = C{twt[2 * t], twt[2 * t + 1]};
+    for (int t = threadIdx.x; t < NP; t += FTHREADS) {
+        if constexpr (sizeof(T) == sizeof(double))  // the FP64 tables hold the twiddles as integers, times 2^62
+            tw[t] = C{(double)__double_as_longlong(twt[2 * t]) * 0x1p-62, (double)__double_as_longlong(twt[2 * t + 1]) * 0x1p-62};
+        else
+            tw[t] = C{twt[2 * t], twt[2 * t + 1]};
+    }
     for (int idx = threadIdx.x; idx < rows * S2 * NP; idx += FTHREADS) {
         const int l = idx % NP, rp = idx / NP, pr = rp % S2, r = rp / S2;
         const T *src = base + (size_t)pr * 2 * blk + (size_t)(i0 + r) * NP + l;

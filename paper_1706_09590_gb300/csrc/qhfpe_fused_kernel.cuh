@@ -19,6 +19,7 @@
 // kernel, and by qhfpe_fused_multi.cu, which instantiates the heterogeneous-batch kernel, so that the
 // two compile in parallel)
 #include "qhfpe.h"
+#include "qhfpe_fixed.cuh"
 #include "qhfpe_internal.cuh"
 
 namespace {
@@ -310,9 +311,11 @@ __device__ __forceinline__ void stv(T *p, const T *in)
 // of different blocks overlapping, and each barrier stalls four warps).  The kernel waits mostly on L2
 // loads, so resident warps count: FP32 with one or two states runs seven blocks per SM (72 registers;
 // measured 5 % faster than six at 80), three states six (seven would spill), NP = 256 four (wider rows).
+// FP64 (integer arithmetic, latency-bound below 16 warps) runs four at 128 registers: on 96 x 128 at depth 8
+// three, four and five blocks took within 3 % of each other, two 25 % longer.
 template <typename T, int NP, int S>
 struct FusedOcc {
-    static constexpr int blocks = sizeof(T) == 4 ? (NP >= 256 ? 4 : (S >= 3 ? 6 : 7)) : 2;
+    static constexpr int blocks = sizeof(T) == 4 ? (NP >= 256 ? 4 : (S >= 3 ? 6 : 7)) : 4;
 };
 
 // Phase A of the fused stage kernels: the potential term of Eq. (quantum-liouvillian) in place on the
@@ -397,6 +400,482 @@ __device__ __forceinline__ void potential_in_place(typename V2<T>::type *X, cons
     fft_all<NP, false>(X, rows * S2, tw);
 }
 
+// Phase A of the FP64 form on block fixed-point integers (qhfpe_fixed.cuh), in place in X: the rows * S^2
+// p-rows as integers of one exponent each, on entry (fill_fixed) and on return.  The same passes as
+// potential_in_place.  The real and imaginary parts of the mixed values are exchanged, which turns the
+// inverse transform into a forward one, so that the radix-16 pass is one function for both directions: with
+// every pass and conversion unrolled twice the instruction cache missed on 39 % of the issue slots.
+// Exponents stand in the padding slots of a transform, as 16-bit values: the row's (before the forward
+// transform, and again after the inverse) at FWD_EXP, those of the runs of 16 modes between at 0 .. R0 - 1.
+template <int NP> struct FixedRows {
+    static constexpr int R0 = Radices<NP>::r[0];
+    static constexpr int PNP = NP + NP / 16;
+    static constexpr int FWD_EXP = R0 == 16 ? 16 : 15;
+    static __device__ __forceinline__ short &exp_slot(double2 *X, int tr, int b)
+    {
+        return reinterpret_cast<short *>(X + tr * PNP + 17 * (b >> 3) + 16)[b & 7];
+    }
+};
+
+// rows * S2 p-rows of the tile into X as integers below 2^bits of their row's exponent
+template <int NP, int S2>
+__device__ __forceinline__ void fill_fixed(double2 *X, const double *__restrict__ v, size_t blk, int i0, int rows)
+{
+    using namespace qhfx;
+    using F = FixedRows<NP>;
+    constexpr int LV = NP >= 128 ? NP / 32 : 4, PL = NP / LV;  // p values per lane, lanes per row
+    constexpr int B = Scale<F::R0>::bits;
+    const int l = (threadIdx.x % PL) * LV;
+#pragma unroll 1
+    for (int base = 0; base < rows * S2; base += FTHREADS / PL) {
+        const int rp = base + threadIdx.x / PL;
+        const bool act = rp < rows * S2;
+        const int pr = act ? rp % S2 : 0, r = act ? rp / S2 : 0;
+        const double *src = v + (size_t)pr * 2 * blk + (size_t)(i0 + r) * NP + l;
+        double re[LV], im[LV];
+        ldv<double, LV>(src, re);
+        ldv<double, LV>(src + blk, im);
+        int E = common_exponent<LV>(re, im);
+#pragma unroll
+        for (int o = PL / 2; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+        if (act) {
+            I2 *x = reinterpret_cast<I2 *>(X + pad16(rp * NP + l));
+#pragma unroll
+            for (int q = 0; q < LV; ++q) x[q] = I2{to_fixed<B>(re[q], E), to_fixed<B>(im[q], E)};
+            if (l == 0) F::exp_slot(X, rp, F::FWD_EXP) = (short)E;
+        }
+    }
+}
+
+// the radix-16 pass over the 16-point runs of n_tr transforms, sign +
+template <int NP> __device__ __noinline__ void pass16_fixed(double2 *X, int n_tr)
+{
+    using namespace qhfx;
+    using F = FixedRows<NP>;
+#pragma unroll 1
+    for (int b = threadIdx.x; b < n_tr * F::R0; b += FTHREADS) {
+        I2 *xb = reinterpret_cast<I2 *>(X) + 17 * b;
+        I2 x[16];
+#pragma unroll
+        for (int t = 0; t < 16; ++t) x[t] = xb[t];
+        dft16<+1>(x);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) xb[t] = x[t];
+    }
+    __syncthreads();
+}
+
+template <int NP, int S>
+__device__ __forceinline__ void potential_fixed(double2 *X, const double2 *tw, const FusedTables<double> &tab, int nq, int i0,
+                                                int rows, double fpp, double ngam, const double *s_lpp, double c2,
+                                                double q_min, double dq)
+{
+    using namespace qhfx;
+    using F = FixedRows<NP>;
+    constexpr int S2 = S * S, R0 = F::R0, PNP = F::PNP;
+    I2 *XI = reinterpret_cast<I2 *>(X);
+    const I2 *w62 = reinterpret_cast<const I2 *>(tw);
+    const int n_tr = rows * S2;
+    const int j = threadIdx.x % 16;  // butterfly of the radix-R0 passes: points j, j + 16, ...
+#pragma unroll 1
+    for (int tr = threadIdx.x / 16; tr < n_tr; tr += FTHREADS / 16) {
+        I2 *xb = XI + tr * PNP + j;
+        I2 x[R0];
+#pragma unroll
+        for (int t = 0; t < R0; ++t) x[t] = xb[17 * t];
+        forward_butterfly<R0>(x, w62, j);
+#pragma unroll
+        for (int u = 0; u < R0; ++u) xb[17 * u] = x[u];
+    }
+    __syncthreads();
+    pass16_fixed<NP>(X, n_tr);
+
+    // mixing: the tables are integers c of one exponent k per pair and row (value c 2^(k - 62)).  A run of 16
+    // modes (a butterfly of the next pass) is brought to the top of the word before the products and again
+    // after their sum, with an exponent of its own: bounds that hold for any row would leave 10 bits unused
+    constexpr int MV = NP > FTHREADS ? 2 : (S == 1 && NP >= 64 ? 2 : 1);  // modes per thread (few: code size)
+    static_assert(FTHREADS % (NP / MV) == 0 && 16 % MV == 0, "mixing positions");
+    constexpr int RS = FTHREADS / (NP / MV);  // rows at once
+    constexpr int RUN = 16 / MV;              // lanes of a run
+    const unsigned run = (RUN == 32 ? 0xffffffffu : ((1u << RUN) - 1)) << (threadIdx.x & 31 & ~(RUN - 1));
+    const int pos0 = (threadIdx.x % (NP / MV)) * MV;
+    const size_t tn = (size_t)nq * NP;
+    const long long *tD = reinterpret_cast<const long long *>(tab.D) + pos0, *tL = reinterpret_cast<const long long *>(tab.L) + pos0,
+                    *tR = reinterpret_cast<const long long *>(tab.R) + pos0;
+    const int *kD = tab.kx, *kL = kD + S2 * nq, *kR = kL + S2 * nq;
+    // the p-diagonal bath terms cf = (f_pp lambda_pp(m) - ngam) / NP, |lambda_pp| <= 64 / NP
+    Half cf[MV];
+    int kcf;
+    const auto bath = [&](double f) {
+        const double bound = (64.0 * fabs(f) + fabs(ngam)) * (1.0 / NP);
+        const int Eb = max(exponent_of(bound) + 1, EXP_MIN);
+        kcf = bound > 0.0 ? Eb - 1022 : -4096;
+#pragma unroll
+        for (int v = 0; v < MV; ++v) cf[v] = halves(to_fixed<62>(f * s_lpp[pos0 + v] - ngam * (1.0 / NP), Eb));
+    };
+    bath(fpp);
+#pragma unroll 1
+    for (int base = 0; base < rows; base += RS) {
+        const int r = base + threadIdx.x / (NP / MV), i = i0 + r;
+        if (r >= rows) break;  // (a run's lanes share their row)
+        if (c2 != 0.0) {       // block-uniform
+            const double ph = 1.0 + 2.0 * c2 * (q_min + i * dq);
+            bath(fpp * ph * ph);
+        }
+        Half xr[S2][MV], xi[S2][MV];
+        int E[S2], big = 0;
+#pragma unroll
+        for (int a = 0; a < S2; ++a) {
+            const int tr = r * S2 + a;
+            E[a] = F::exp_slot(X, tr, F::FWD_EXP);
+            big = max(big, E[a]);
+            I2 q[MV];
+            unsigned o = 0;
+#pragma unroll
+            for (int v = 0; v < MV; ++v) {
+                q[v] = XI[tr * PNP + pad16(pos0 + v)];
+                o |= magnitude(q[v]);
+            }
+            const int n = norm_shift<61>(__reduce_or_sync(run, o));
+            E[a] -= n;
+#pragma unroll
+            for (int v = 0; v < MV; ++v) {
+                q[v] = shift(q[v], n);
+                xr[a][v] = halves(q[v].x);
+                xi[a][v] = halves(q[v].y);
+            }
+        }
+#pragma unroll
+        for (int j_ = 0; j_ < S; ++j_)
+#pragma unroll
+            for (int k = 0; k < S; ++k) {
+                const int jk = j_ * S + k;
+                int M = max(E[jk] + kD[jk * nq + i], E[jk] + kcf);
+#pragma unroll
+                for (int s = 0; s < S; ++s) {
+                    if (s != j_) M = max(M, E[s * S + k] + kL[(j_ * S + s) * nq + i]);
+                    if (s != k) M = max(M, E[j_ * S + s] + kR[(s * S + k) * nq + i]);
+                }
+                M = max(M, 100);
+                long long ar[MV], ai[MV];  // the commutator: at most six products below 2^60
+                {
+                    const int sh = M - (E[jk] + kD[jk * nq + i]);
+#pragma unroll
+                    for (int v = 0; v < MV; ++v) {
+                        const Half c = halves(tD[jk * tn + (size_t)i * NP + v]);
+                        ar[v] = shr_s(mul_hi(xr[jk][v], c), sh);
+                        ai[v] = shr_s(mul_hi(xi[jk][v], c), sh);
+                    }
+                }
+#pragma unroll
+                for (int s = 0; s < S; ++s) {
+                    if (s != j_) {
+                        const int a = s * S + k, t = j_ * S + s, sh = M - (E[a] + kL[t * nq + i]);
+#pragma unroll
+                        for (int v = 0; v < MV; ++v) {
+                            const Half c = halves(tL[t * tn + (size_t)i * NP + v]);
+                            ar[v] += shr_s(mul_hi(xr[a][v], c), sh);
+                            ai[v] += shr_s(mul_hi(xi[a][v], c), sh);
+                        }
+                    }
+                    if (s != k) {
+                        const int a = j_ * S + s, t = s * S + k, sh = M - (E[a] + kR[t * nq + i]);
+#pragma unroll
+                        for (int v = 0; v < MV; ++v) {
+                            const Half c = halves(tR[t * tn + (size_t)i * NP + v]);
+                            ar[v] -= shr_s(mul_hi(xr[a][v], c), sh);
+                            ai[v] -= shr_s(mul_hi(xi[a][v], c), sh);
+                        }
+                    }
+                }
+                const int sc = M - (E[jk] + kcf), tr = r * S2 + jk;
+                I2 q[MV];
+                unsigned o = 0;
+#pragma unroll
+                for (int v = 0; v < MV; ++v) {  // times -i, plus the bath terms; parts exchanged
+                    q[v] = I2{shr_s(mul_hi(xi[jk][v], cf[v]), sc) - ar[v], shr_s(mul_hi(xr[jk][v], cf[v]), sc) + ai[v]};
+                    o |= magnitude(q[v]);
+                }
+                const int n = norm_shift<59>(__reduce_or_sync(run, o));
+#pragma unroll
+                for (int v = 0; v < MV; ++v) XI[tr * PNP + pad16(pos0 + v)] = shift(q[v], n);
+                if (pos0 % 16 == 0) F::exp_slot(X, tr, pos0 / 16) = (short)(big >= EXP_BIG ? EXP_BIG : min(M - n, EXP_BIG));
+            }
+    }
+    __syncthreads();
+    pass16_fixed<NP>(X, n_tr);
+#pragma unroll 1
+    for (int tr = threadIdx.x / 16; tr < n_tr; tr += FTHREADS / 16) {
+        I2 *xb = XI + tr * PNP + j;
+        I2 x[R0];
+        int e[R0];
+#pragma unroll
+        for (int t = 0; t < R0; ++t) {
+            x[t] = xb[17 * t];
+            e[t] = F::exp_slot(X, tr, t);
+        }
+        const int E = align<R0>(x, e);
+        inverse_butterfly<R0>(x, w62, j);
+#pragma unroll
+        for (int t = 0; t < R0; ++t) xb[17 * t] = I2{x[t].y, x[t].x};
+        if (j == 0) F::exp_slot(X, tr, F::FWD_EXP) = (short)E;
+    }
+    __syncthreads();
+}
+// the potential term in X is v 2^(E + fixed_pot_exponent), E at the transform's FWD_EXP (EXP_BIG: NaN)
+template <int NP, int S> constexpr int fixed_pot_exponent()
+{
+    constexpr int R0 = Radices<NP>::r[0];
+    return qhfx::Scale<R0>::K_fwd + 4 + 2 + qhfx::Scale<R0>::inv + qhfx::Scale<R0>::down;
+}
+// ... as doubles, for the phase B in FP64
+template <int NP, int S> __device__ __forceinline__ void potential_to_double(double2 *X, int n_tr)
+{
+    using namespace qhfx;
+    for (int t = threadIdx.x; t < n_tr * NP; t += FTHREADS) {
+        const int tr = t / NP, M = FixedRows<NP>::exp_slot(X, tr, FixedRows<NP>::FWD_EXP);
+        const I2 v = reinterpret_cast<const I2 *>(X)[pad16(t)];
+        const double bad = bitsd(0x7ff8000000000000ull);
+        const int K = M + fixed_pot_exponent<NP, S>();
+        X[pad16(t)] = M >= EXP_BIG ? double2{bad, bad} : double2{from_fixed(v.x, K), from_fixed(v.y, K)};
+    }
+}
+
+// A tier coupling's weight for the fixed-point sums: w = c 2^(k - 62), |c| in [2^61, 2^62).
+struct FixedWeight {
+    qhfx::Half c;
+    int k;
+};
+__device__ __forceinline__ FixedWeight fixed_weight(double w)
+{
+    const int ex = qhfx::exponent_of(w);
+    if (ex == 0) return FixedWeight{{0, 0}, -4096};  // far below every other term
+    const long long m = qhfx::to_fixed<62>(w, ex);
+    return FixedWeight{qhfx::halves(m), ex - 1022};
+}
+constexpr int FIXED_MAXNB = 12;  // terms of a tier sum: 12 x 18 x 2^55 stays below 2^63
+
+// Phase B of the FP64 form (linear coupling, all terms, the potential and the p-diagonal bath terms already
+// in X): kinetic term, tier couplings and update of the block's rows.  As in the transforms
+// (qhfpe_fixed.cuh) the FP64 pipe would bound it, so the sums run on 64-bit integers:
+//   kinetic  the q differences have small integer weights (sum of sizes 130).  A warp takes four rows of one
+//            pair; for each of its p columns the nine rows read are brought to the column's largest exponent
+//            (62 bits below it) once, and the four sums of six are exact.  Where the rows' own exponents are
+//            more than eight apart each of the four takes its own.
+//   tiers    G = sum of the neighbours' rows, weighted; every term (value times weight) is brought to the row's
+//            largest exponent, 55 bits below it, and the p difference of G (weights 1, 8) is exact.
+// Quantising at 2^-54 to 2^-62 of the largest term is below the rounding of the FP64 sums, whose partial sums of
+// up to 100 times the values round at 2^-53.  Three FP64 instructions per value remain (the scaled p difference,
+// p W^(n-e_0), out = y + h L) of 43.
+// Infinities, NaN and values from 2^1007: a column or row that holds one gives NaN.
+template <int NP, int S>
+__device__ __forceinline__ void
+rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__restrict__ v_in, const double *y, double *v_out,
+           int mode, size_t ebase, int i0, int rows, const long long *nb_off, const FixedWeight *nb_fw, const double *nb_wa,
+           int n_up, int n_d0, int n_nb, bool term, double2 *X, const double *pgrid)
+{
+    using namespace qhfx;
+    constexpr int S2 = S * S;
+    constexpr int VEC = NP / 32;              // a warp holds a p row
+    constexpr int RG = 4;                     // q rows per unit
+    constexpr int BITS = 55;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t blk = g.blk;
+    const int nq = g.nq;
+    const int l0 = lane * VEC;
+    const bool neg = pgrid[l0] < 0.0;  // one sign per lane (caller's check)
+    int ck[6];                         // p < 0: offsets -2..+3, p >= 0: -3..+2
+    {
+        const int cneg[6] = {3, -30, -20, 60, -15, 2}, cpos[6] = {-2, 15, -60, 20, 30, -3};
+#pragma unroll
+        for (int t = 0; t < 6; ++t) ck[t] = neg ? cneg[t] : cpos[t];
+    }
+    const int first = neg ? -2 : -3;
+    const double bad = bitsd(0x7ff8000000000000ull);
+#pragma unroll 1
+    for (int u = warp; u < ((rows + RG - 1) / RG) * S2; u += FTHREADS / 32) {
+        const int pr = u % S2, r0 = (u / S2) * RG;
+        const int nr = min(RG, rows - r0);
+        const int ia = i0 + r0;
+        const size_t poff = ebase + (size_t)pr * 2 * blk;
+#pragma unroll 1
+        for (int plane = 0; plane < 2; ++plane) {
+            const double *V = v_in + poff + plane * blk;
+            // (each lane reads and writes only its own values of X from here on)
+            const auto Xat = [&](int r, int v) -> double & {
+                return reinterpret_cast<double *>(X + pad16(((r0 + r) * S2 + pr) * NP + l0 + v))[plane];
+            };
+#pragma unroll 1
+            for (int v = 0; v < VEC; ++v) {  // (one p column at a time: more in flight would only lengthen the code)
+                const FixedWeight pk = fixed_weight(-(pgrid[l0 + v] * sc.fkin));
+                const auto value = [&](int t) {  // window row t of the column
+                    int ii = ia + first + t;
+                    bool ok = t < nr + 5 && ii >= 0 && ii < nq;
+                    if (!ok && g.periodic_q && t < nr + 5) {
+                        ii = ii < 0 ? ii + nq : ii - nq;
+                        ok = ii >= 0 && ii < nq;
+                    }
+                    return ok ? V[(size_t)ii * NP + l0 + v] : 0.0;
+                };
+                // row r from its six window rows x (below 2^62) of exponent E: -p dW/dq and the potential term, each
+                // an integer, at the larger unit
+                const auto emit = [&](int r, const Half *x, int E) {
+                    long long lo = 0, hi = 0;
+#pragma unroll
+                    for (int t = 0; t < 6; ++t) {
+                        lo = madw(x[t].l, ck[t], lo);
+                        hi = madw(x[t].h, ck[t], hi);
+                    }
+                    const long long kin = mul_hi(halves((long long)((unsigned long long)hi << 24) + (lo >> 8)), pk.c);
+                    double &xv = Xat(r, v);
+                    const long long pot = (long long)dbits(xv);
+                    const int M = FixedRows<NP>::exp_slot(X, (r0 + r) * S2 + pr, FixedRows<NP>::FWD_EXP);
+                    const int uk = E + pk.k - 1022 - 62 + 8 + 2, up = M + fixed_pot_exponent<NP, S>();
+                    const int U = max(max(uk, up), -1000);  // (below 2^60 and 2^62: the sum fits)
+                    const long long fine = uk < up ? kin : pot, coarse = uk < up ? pot : kin;
+                    const double a = from_fixed(shr_round(coarse, U - max(uk, up)) + shr_round(fine, U - min(uk, up)), U);
+                    xv = E >= EXP_BIG || M >= EXP_BIG ? bad : a;
+                };
+                double raw[RG + 5];
+                int ex[RG + 5], E = EXP_MIN;
+#pragma unroll
+                for (int t = 0; t < RG + 5; ++t) raw[t] = value(t);
+#pragma unroll
+                for (int t = 0; t < RG + 5; ++t) {
+                    ex[t] = exponent_of(raw[t]);
+                    E = max(E, ex[t]);
+                }
+                int least = E;  // smallest of the rows' own exponents
+#pragma unroll
+                for (int r = 0; r < RG; ++r) {
+                    const int er = max(max(max(ex[r], ex[r + 1]), max(ex[r + 2], ex[r + 3])), max(ex[r + 4], ex[r + 5]));
+                    if (r < nr) least = min(least, er);
+                }
+                if (!__any_sync(0xffffffffu, E - least > 8)) {
+                    Half x[RG + 5];
+#pragma unroll
+                    for (int t = 0; t < RG + 5; ++t) x[t] = halves(to_fixed<62>(raw[t], E));
+#pragma unroll
+                    for (int r = 0; r < RG; ++r)
+                        if (r < nr) emit(r, x + r, E);
+                } else {  // steep in q: an exponent for each row
+#pragma unroll 1
+                    for (int r = 0; r < nr; ++r) {
+                        Half x[6];
+                        double w[6];
+                        int er = EXP_MIN;
+#pragma unroll
+                        for (int t = 0; t < 6; ++t) {
+                            w[t] = value(r + t);
+                            er = max(er, exponent_of(w[t]));
+                        }
+#pragma unroll
+                        for (int t = 0; t < 6; ++t) x[t] = halves(to_fixed<62>(w[t], er));
+                        emit(r, x, er);
+                    }
+                }
+            }
+            double p[VEC], pw[VEC];  // p, and times the weight of the (first) neighbour with a p term
+            ldv<double, VEC>(pgrid + l0, p);
+            if (n_d0 < n_nb) {
+                const double wa = nb_wa[n_d0];
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) pw[v] = p[v] * wa;
+            }
+#pragma unroll 1
+            for (int r = 0; r < nr; ++r) {
+                const int i = ia + r;
+                const size_t o = poff + plane * blk + (size_t)i * NP + l0;
+                double a[VEC];
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) a[v] = Xat(r, v);  // potential and kinetic terms
+                // G at the row's exponent E, built up term by term
+                long long G[VEC];
+                int E = EXP_MIN;
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) G[v] = 0;
+                // the neighbours in turn, the next one's values in flight; last the terminator's r_0 p W
+                const int n_terms = n_nb + (term ? 1 : 0);
+                const auto source = [&](int n) { return v_in + (long long)o + (n < n_nb ? nb_off[n] : 0); };
+                double next[VEC];
+                if (n_terms > 0) ldv<double, VEC>(source(0), next);
+#pragma unroll 1
+                for (int n = 0; n < n_terms; ++n) {
+                    double w[VEC];
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) w[v] = next[v];
+                    if (n + 1 < n_terms) ldv<double, VEC>(source(n + 1), next);
+                    if (n >= n_d0) {  // warp-uniform; (the barrier keeps it a branch: FP64 instructions that
+                                      // are only predicated off take their 64 clocks all the same)
+                        __syncwarp();
+                        if (n >= n_nb) {
+#pragma unroll
+                            for (int v = 0; v < VEC; ++v) w[v] *= sc.r0 * p[v];
+                        } else {
+                            const double wa = nb_wa[n];
+#pragma unroll
+                            for (int v = 0; v < VEC; ++v) a[v] = fma(n == n_d0 ? pw[v] : p[v] * wa, w[v], a[v]);
+                        }
+                    }
+                    const bool weighted = n >= n_up && n < n_nb;
+                    const FixedWeight fw = nb_fw[n < FIXED_MAXNB ? n : 0];
+                    const int k = weighted ? fw.k : 0;
+                    int em = 0;
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) em = max(em, exponent_of(w[v]));
+                    em = em >= EXP_BIG ? 2 * EXP_BIG : em + k;
+                    em = __reduce_max_sync(0xffffffffu, em);
+                    if (em > E) {  // warp-uniform
+#pragma unroll
+                        for (int v = 0; v < VEC; ++v) G[v] = shr_s(G[v], em - E);
+                        E = em;
+                    }
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) {
+                        const long long x = to_fixed<BITS + 2>(w[v], E - k);
+                        if (weighted) {
+                            G[v] += mul_hi(halves(x), fw.c);
+                        } else {
+                            G[v] += x >> 2;
+                        }
+                    }
+                }
+                if (n_nb > 0 || term) {  // 4th-order central d/dp of G, periodic p, neighbours through the warp
+                    long long e[VEC + 4];
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) e[v + 2] = G[v];
+                    const unsigned all = 0xffffffffu;
+                    if constexpr (VEC == 1) {
+                        e[0] = __shfl_sync(all, G[0], (lane + 30) & 31);
+                        e[1] = __shfl_sync(all, G[0], (lane + 31) & 31);
+                        e[3] = __shfl_sync(all, G[0], (lane + 1) & 31);
+                        e[4] = __shfl_sync(all, G[0], (lane + 2) & 31);
+                    } else {
+                        e[0] = __shfl_sync(all, G[VEC - 2], (lane + 31) & 31);
+                        e[1] = __shfl_sync(all, G[VEC - 1], (lane + 31) & 31);
+                        e[VEC + 2] = __shfl_sync(all, G[0], (lane + 1) & 31);
+                        e[VEC + 3] = __shfl_sync(all, G[1], (lane + 1) & 31);
+                    }
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) {
+                        const long long d = (e[v] - e[v + 4]) + ((e[v + 3] - e[v + 1]) << 3);
+                        double dg = from_fixed(d, E - 1022 - BITS);
+                        if (E >= EXP_BIG) dg = bad;
+                        a[v] = fma(sc.inv12dp, dg, a[v]);
+                    }
+                }
+                if (mode != 0) {
+                    double b[VEC];
+                    ldv<double, VEC>(y + o, b);
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) a[v] = fma(sc.h, a[v], b[v]);
+                }
+                stv<double, VEC>(v_out + o, a);
+            }
+        }
+    }
+}
+
 // MULTI: one Horner stage of several propagators at once (heterogeneous batch: members differ in q
 // grid, surfaces, bath, hierarchy depth, closure, dt and replica count, and share NP, S and the
 // precision).  Blocks are numbered member by member; a block finds its member (first block numbers
@@ -473,6 +952,7 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
 
     __shared__ long long nb_off[3 * QH_MAX_MODES];
     __shared__ T nb_wg[3 * QH_MAX_MODES], nb_wa[3 * QH_MAX_MODES];
+    __shared__ FixedWeight nb_fw[FIXED_MAXNB];  // FP64 form: nb_wg for the fixed-point sums
     __shared__ long long mx_off[QH_MAX_MODES];  // nonlinear coupling: mixed-derivative neighbours
     __shared__ T mx_w[QH_MAX_MODES];
     __shared__ int s_nmx;
@@ -518,6 +998,21 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
         s_cnt[3] = (terms & 8) && E.terminator;
         s_ngam = (terms & 4) ? (T)E.ngam : (T)0;
     }
+    if constexpr (sizeof(T) == sizeof(double) && !NL) {
+        // (read after the barriers of phase A)
+        if (threadIdx.x >= 32 && threadIdx.x < 32 + FIXED_MAXNB) {
+            const ElemInfo &E = elems[e];
+            const int a = threadIdx.x - 32;
+            // the order of nb_wg: up, down without a p term, down with one
+            int n = E.n_up;
+            for (int pass = 0; pass < 2; ++pass)
+                for (int d = 0; d < E.n_dn; ++d)
+                    if ((E.wr[d] != 0.0) == (pass == 1)) {
+                        if (n == a) nb_fw[a] = fixed_weight(E.wc[d]);
+                        ++n;
+                    }
+        }
+    }
     if (!warm)
         for (int t = threadIdx.x; t < NP; t += FTHREADS) {
             tw[t] = C{tab.tw[2 * t], tab.tw[2 * t + 1]};
@@ -535,7 +1030,15 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
     // terminator are circulants along p, i.e. products with their eigenvalues after the FFT.
     const bool want_pot = (terms & 2) != 0;
     const bool fold = want_pot && !Pg;
-    if (fold) {
+    if constexpr (sizeof(T) == sizeof(double)) {
+        if (fold) {
+            fill_fixed<NP, S2>(X, v_in + ebase, blk, i0, rows);
+            __syncthreads();
+            potential_fixed<NP, S>(X, tw, tab, nq, i0, rows,
+                                   ((terms & 4) ? sc.fdelta : (T)0) + ((s_cnt[3] != 0) ? sc.fterm : (T)0), s_ngam, s_lpp,
+                                   NL ? g.c2 : 0.0, g.q_min, g.dq);
+        }
+    } else if (fold) {
         constexpr int LV = 4;  // p values per load
         constexpr int PL = NP / LV;
         static_assert(FTHREADS % PL == 0, "load positions");
@@ -574,6 +1077,21 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
     const bool uni_warp = __all_sync(0xffffffffu, neg0 == (pcol[VEC - 1] < (T)0));
     const int sh = neg0 ? 1 : 0;
     const bool interior = i0 >= 3 && i0 + rows + 3 <= nq;  // no q-stencil row outside the grid
+    if constexpr (sizeof(T) == sizeof(double) && !NL) {
+        // the fixed-point form: all terms, the potential in X, every lane's p values of one sign
+        const bool one_sign = __all_sync(0xffffffffu, (pgrid[lane * (NP / 32)] < (T)0) == (pgrid[lane * (NP / 32) + NP / 32 - 1] < (T)0));
+        if (fold && terms == QHFPE_TERM_ALL && one_sign && n_nb + (term ? 1 : 0) <= FIXED_MAXNB) {
+            rows_fixed<NP, S>(g, sc, v_in, y, v_out, mode, ebase, i0, rows, nb_off, nb_fw, nb_wa, n_up, n_d0, n_nb, term, X,
+                              pgrid);
+            return;
+        }
+    }
+    if constexpr (sizeof(T) == sizeof(double)) {
+        if (fold) {
+            potential_to_double<NP, S>(X, rows * S2);
+            __syncthreads();
+        }
+    }
     T pk[VEC];  // -p / (60 dq)
 #pragma unroll
     for (int v = 0; v < VEC; ++v) pk[v] = -(pcol[v] * fkin);

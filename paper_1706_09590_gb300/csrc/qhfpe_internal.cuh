@@ -66,11 +66,15 @@ struct PotTables {
 // Tables of the fused stage kernel: same D, L, R as PotTables but in the fused FFT's
 // digit-reversed order (fused_fft_frequency), np twiddles e^{2 pi i t/np}, t < np, and lpp: the
 // eigenvalues of the periodic 5-point d2/dp2 stencil (without 1/(12 dp^2)) at each FFT position, over np.
+// The FP64 form's transforms and mixing run on integers (qhfpe_fixed.cuh): its D, L, R and tw hold 64-bit
+// integers in the places of the doubles, twiddles times 2^62 and table values times 2^(62 - k) with the
+// exponents k of each table, pair and q row in kx [3][S][S][nq] (nullptr in FP32).
 template <typename T>
 struct FusedTables {
     const T *D, *L, *R;
     const T *tw;
     const T *lpp;
+    const int *kx;
 };
 
 // Scalars of one fused stage launch, rounded once on the host: 1/(12 dp), 1/(60 dq), the delta-term and
