@@ -834,7 +834,7 @@ qhfpe_status autotune(qhfpe *h, Prop &P)
     float best = 1e30f, ms = 0.f;
     int best_tq = 1, best_form = 0;
     // the kernel form: the q-window kernel (fixed tile) where it applies, against the general kernel
-    if (P.mixed && !P.tc && fused_window_applies(P.g, QHFPE_TERM_ALL, false)) {
+    if (P.mixed && fused_window_applies(P.g, QHFPE_TERM_ALL)) {
         qhfpe_status r = time_one(1, 0, &ms);
         if (r != QHFPE_OK) return r;
         best = ms;
@@ -2045,7 +2045,7 @@ qhfpe_status qhfpe_stage_form(const qhfpe_t *h, int *form)
     const Prop &P = *h->main;
     if (!P.tq) *form = -1;
     else if (P.form >= 0) *form = P.form;
-    else *form = (P.mixed && !P.tc && fused_window_applies(P.g, QHFPE_TERM_ALL, false)) ? 1 : 0;  // pinned tile
+    else *form = (P.mixed && fused_window_applies(P.g, QHFPE_TERM_ALL)) ? 1 : 0;  // pinned tile
     return QHFPE_OK;
 }
 

@@ -104,7 +104,7 @@ cudaError_t launch_dipole_fft_t(const GridInfo &g, const T *TL, const T *TR, con
 }
 
 // The q-window kernel serves FP32 states with np = 128 and one or two electronic states when the stage
-// computes every term with the potential term in the kernel, each lane's four p values share a sign
+// computes every term (the potential term itself, or from the tensor-core kernel), each lane's four p values share a sign
 // (p = 0 on a multiple of four, or off the grid), and no element has more than six tier neighbours.
 // QHFPE_FUSED_WINDOW=0 in the environment selects fused_stage_kernel instead.
 bool window_enabled()
@@ -117,10 +117,10 @@ bool window_enabled()
 
 int fused_window_rows(int S) { return S == 1 ? WinTile<1>::TQ : WinTile<2>::TQ; }
 
-bool fused_window_applies(const GridInfo &g, int terms, bool have_pg)
+bool fused_window_applies(const GridInfo &g, int terms)
 {
     const int np = g.np, S = g.S;
-    if (np != 128 || S < 1 || S > 2 || have_pg || terms != QHFPE_TERM_ALL || g.max_nb > WIN_MAXNB || g.c2 != 0.0)
+    if (np != 128 || S < 1 || S > 2 || terms != QHFPE_TERM_ALL || g.max_nb > WIN_MAXNB || g.c2 != 0.0)
         return false;
     for (int c = 0; c < np; c += 4) {
         const bool a = (float)(g.p_min + c * g.dp) < 0.0f, b = (float)(g.p_min + (c + 3) * g.dp) < 0.0f;
@@ -131,13 +131,13 @@ bool fused_window_applies(const GridInfo &g, int terms, bool have_pg)
 
 namespace {
 
-template <int S, bool MIXED>
+template <int S, bool MIXED, bool PG>
 cudaError_t launch_window_t(const GridInfo &g, const ElemInfo *elems, const FusedTables<float> &tab, const float *v_in,
                             const float *y, const double *y0, float *v_out, double *y0_out, double h, int mode,
-                            int rep0, int n_rep, cudaStream_t st)
+                            int rep0, int n_rep, cudaStream_t st, const float *Pg)
 {
     constexpr int NP = 128, TQ = WinTile<S>::TQ;
-    const size_t smem = win_kin_offset<NP, S, TQ>() + WIN_KIN_BYTES;
+    const size_t smem = win_smem<NP, S, TQ, PG>();
     const long blocks = (long)((g.nq + TQ - 1) / TQ) * n_rep * g.n_elem;
     if (blocks <= 0) return cudaSuccess;
     const StageScalars<float> sc = stage_scalars<float>(g, h);
@@ -151,8 +151,8 @@ cudaError_t launch_window_t(const GridInfo &g, const ElemInfo *elems, const Fuse
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fused_window_kernel<NP, S, MIXED>, g, elems, tab, sc, v_in, y, y0, v_out, y0_out, h,
-                              mode, rep0, n_rep);
+    return cudaLaunchKernelEx(&cfg, fused_window_kernel<NP, S, MIXED, PG>, g, elems, tab, sc, v_in, y, y0, v_out, y0_out,
+                              h, mode, rep0, n_rep, Pg);
 }
 
 template <typename T, int NP, int S, bool MIXED>
@@ -161,8 +161,9 @@ cudaError_t launch_fused_t(const GridInfo &g, const ElemInfo *elems, const Fused
                            int rep0, int n_rep, cudaStream_t st, const T *Pg, int tq_req, int form)
 {
     if constexpr (sizeof(T) == 4 && NP == 128 && S <= 2) {
-        if (form != 0 && fused_window_applies(g, terms, Pg != nullptr))
-            return launch_window_t<S, MIXED>(g, elems, tab, v_in, y, y0, v_out, y0_out, h, mode, rep0, n_rep, st);
+        if (form != 0 && fused_window_applies(g, terms))
+            return Pg ? launch_window_t<S, MIXED, true>(g, elems, tab, v_in, y, y0, v_out, y0_out, h, mode, rep0, n_rep, st, Pg)
+                      : launch_window_t<S, MIXED, false>(g, elems, tab, v_in, y, y0, v_out, y0_out, h, mode, rep0, n_rep, st, Pg);
     }
     if (g.c2 != 0.0)  // the nonlinear coupling's terms: the instantiation of qhfpe_fused_nl.cu
         return launch_fused_nl<T, MIXED>(g, elems, tab, v_in, y, y0, v_out, y0_out, h, mode, terms, rep0, n_rep, st, Pg,
@@ -182,8 +183,11 @@ cudaError_t prepare_fused_t()
     if (e != cudaSuccess) return e;
     if constexpr (sizeof(T) == 4 && NP == 128 && S <= 2) {
         constexpr int TQ = WinTile<S>::TQ;
-        e = cudaFuncSetAttribute(fused_window_kernel<NP, S, MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(win_kin_offset<NP, S, TQ>() + WIN_KIN_BYTES));
+        e = cudaFuncSetAttribute(fused_window_kernel<NP, S, MIXED, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)win_smem<NP, S, TQ, false>());
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(fused_window_kernel<NP, S, MIXED, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)win_smem<NP, S, TQ, true>());
         if (e != cudaSuccess) return e;
     }
     return prepare_fused_multi<T, MIXED>(NP, S, smem);

@@ -16,7 +16,7 @@
 // The kinetic term of the unit's rows waits in shared memory (each lane reads back only what it wrote)
 // so that no registers are held across phase A.
 // Requirements (checked by the launcher): every lane's four p values have one sign, at most six tier
-// neighbours per element, the potential term computed here (all terms).
+// neighbours per element, all terms.
 #pragma once
 #include "qhfpe_fused_kernel.cuh"
 
@@ -38,11 +38,21 @@ __host__ __device__ constexpr size_t win_kin_offset()
 }
 constexpr size_t WIN_KIN_BYTES = (FTHREADS / 32) * WIN_RG * 2 * 128 * sizeof(float);
 
-template <int NP, int S, bool MIXED>
+// dynamic shared memory: the FFT buffer and twiddles (absent when the potential term comes from another
+// kernel), then the kinetic terms
+template <int NP, int S, int TQ, bool PG> constexpr size_t win_smem()
+{
+    return (PG ? 0 : win_kin_offset<NP, S, TQ>()) + WIN_KIN_BYTES;
+}
+
+// PG: the potential term is read from Pg (the tensor-core form); phase A is left out, and the p-diagonal
+// bath terms are applied to the centre row instead of in r-space.  On 96 x 128 at depth 8 the tensor-core form's
+// step went from 0.699 to 0.680 ms (general kernel to this one).
+template <int NP, int S, bool MIXED, bool PG>
 __global__ void __launch_bounds__(FTHREADS, WIN_BLOCKS)
 fused_window_kernel(GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<float> tab, StageScalars<float> sc,
                     const float *__restrict__ v_in, const float *y, const double *y0, float *v_out, double *y0_out,
-                    double h, int mode, int rep0, int n_rep)
+                    double h, int mode, int rep0, int n_rep, const float *__restrict__ Pg)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     using T = float;
@@ -97,9 +107,11 @@ fused_window_kernel(GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<
         s_ngam = (T)E.ngam;
     }
     for (int t = threadIdx.x; t < NP; t += FTHREADS) {
-        tw[t] = C{tab.tw[2 * t], tab.tw[2 * t + 1]};
+        if (!PG) {
+            tw[t] = C{tab.tw[2 * t], tab.tw[2 * t + 1]};
+            s_lpp[t] = tab.lpp[t];
+        }
         pgrid[t] = (T)(g.p_min + t * g.dp);
-        s_lpp[t] = tab.lpp[t];
     }
     __syncthreads();
 
@@ -126,7 +138,7 @@ fused_window_kernel(GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     const size_t poff = ebase + (size_t)pr * 2 * blk;
-    float *kbuf = reinterpret_cast<float *>(smem_raw + win_kin_offset<NP, S, TQ>()) + (size_t)warp * RG * 2 * NP;
+    float *kbuf = reinterpret_cast<float *>(smem_raw + (PG ? 0 : win_kin_offset<NP, S, TQ>())) + (size_t)warp * RG * 2 * NP;
 
     // ---- 1. window: kinetic term of the unit's rows, own rows into the FFT buffer ------------------
     const T *Vre = v_in + poff, *Vim = Vre + blk;
@@ -168,7 +180,7 @@ fused_window_kernel(GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<
                     v_axpy<VEC>(ki[r], ck[tap], wi_[b]);
                 }
             }
-            if (t >= 3 && t < 3 + RG) {  // an own row: into the FFT buffer (rows past the grid are zero)
+            if (!PG && t >= 3 && t < 3 + RG) {  // an own row: into the FFT buffer (rows past the grid are zero)
                 const int lr = rg * RG + t - 3;
                 C *xb = X + pad16((lr * S2 + pr) * NP + l0);
 #pragma unroll
@@ -188,16 +200,19 @@ fused_window_kernel(GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<
     }
 
     // ---- 2. phase A: potential term and the p-diagonal bath terms, in place in X ------------------
-    __syncthreads();
-    potential_in_place<T, NP, S>(X, tw, tab, nq, i0, rows, sc.fdelta + (s_cnt[3] != 0 ? sc.fterm : (T)0), s_ngam,
-                                 s_lpp);
+    const T fpp = sc.fdelta + (s_cnt[3] != 0 ? sc.fterm : (T)0), ngam = s_ngam;
+    if constexpr (!PG) {
+        __syncthreads();
+        potential_in_place<T, NP, S>(X, tw, tab, nq, i0, rows, fpp, ngam, s_lpp);
+    }
 
     // ---- 3. per q row: tier couplings, p-stencil, update -------------------------------------------
     const int n_up = s_cnt[0], n_d0 = s_cnt[1], n_nb = s_cnt[2];
     const bool term = s_cnt[3] != 0;
     const T inv12dp = sc.inv12dp;
     const bool tier0 = MIXED && e == 0;
-#pragma unroll
+    constexpr int UNROLL = PG ? 1 : RG;  // (PG: spills when unrolled)
+#pragma unroll UNROLL
     for (int r = 0; r < RG; ++r) {
         const int i = ia + r;
         if (i >= nq || i >= i0 + rows) continue;  // warp-uniform
@@ -253,38 +268,62 @@ fused_window_kernel(GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<
             v_fma<VEC>(ar, pcol, hr);
             v_fma<VEC>(ai, pcol, hi);
         }
-        if (term) {  // d/dp (r_0 p W) of the Eq. (GMFP) terminator: the centre row again
+        // a row's values with two neighbours on each side (periodic p), through the warp
+        const auto widen = [&](const T *xr, const T *xi, T *er, T *ei) {
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) {
+                er[v + 2] = xr[v];
+                ei[v + 2] = xi[v];
+            }
+            const int left = (lane + 31) & 31, right = (lane + 1) & 31;
+            er[0] = __shfl_sync(0xffffffffu, xr[VEC - 2], left);
+            er[1] = __shfl_sync(0xffffffffu, xr[VEC - 1], left);
+            ei[0] = __shfl_sync(0xffffffffu, xi[VEC - 2], left);
+            ei[1] = __shfl_sync(0xffffffffu, xi[VEC - 1], left);
+            er[VEC + 2] = __shfl_sync(0xffffffffu, xr[0], right);
+            er[VEC + 3] = __shfl_sync(0xffffffffu, xr[1], right);
+            ei[VEC + 2] = __shfl_sync(0xffffffffu, xi[0], right);
+            ei[VEC + 3] = __shfl_sync(0xffffffffu, xi[1], right);
+        };
+        if (PG || term) {  // the centre row again
             T wr[VEC], wi[VEC], r0p[VEC];
             ldv<T, VEC>(Vre + (size_t)i * NP + l0, wr);
             ldv<T, VEC>(Vim + (size_t)i * NP + l0, wi);
+            if (term) {  // d/dp (r_0 p W) of the Eq. (GMFP) terminator
 #pragma unroll
-            for (int v = 0; v < VEC; ++v) r0p[v] = sc.r0 * pcol[v];
-            v_fma<VEC>(gr, r0p, wr);
-            v_fma<VEC>(gi, r0p, wi);
-        }
-        if (n_nb > 0 || term) {  // 4th-order central d/dp of G, periodic p, neighbours through the warp
-            T er[VEC + 4], ei[VEC + 4];
-#pragma unroll
-            for (int v = 0; v < VEC; ++v) {
-                er[v + 2] = gr[v];
-                ei[v + 2] = gi[v];
+                for (int v = 0; v < VEC; ++v) r0p[v] = sc.r0 * pcol[v];
+                v_fma<VEC>(gr, r0p, wr);
+                v_fma<VEC>(gi, r0p, wi);
             }
-            const int left = (lane + 31) & 31, right = (lane + 1) & 31;
-            er[0] = __shfl_sync(0xffffffffu, gr[VEC - 2], left);
-            er[1] = __shfl_sync(0xffffffffu, gr[VEC - 1], left);
-            ei[0] = __shfl_sync(0xffffffffu, gi[VEC - 2], left);
-            ei[1] = __shfl_sync(0xffffffffu, gi[VEC - 1], left);
-            er[VEC + 2] = __shfl_sync(0xffffffffu, gr[0], right);
-            er[VEC + 3] = __shfl_sync(0xffffffffu, gr[1], right);
-            ei[VEC + 2] = __shfl_sync(0xffffffffu, gi[0], right);
-            ei[VEC + 3] = __shfl_sync(0xffffffffu, gi[1], right);
+            if constexpr (PG) {  // damping, delta-term and the terminator's d2/dp2, and the potential term
+                v_axpy<VEC>(ar, -ngam, wr);
+                v_axpy<VEC>(ai, -ngam, wi);
+                if (fpp != (T)0) {
+                    T er[VEC + 4], ei[VEC + 4];
+                    widen(wr, wi, er, ei);
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) {
+                        ar[v] += fpp * (-er[v] + (T)16 * er[v + 1] - (T)30 * er[v + 2] + (T)16 * er[v + 3] - er[v + 4]);
+                        ai[v] += fpp * (-ei[v] + (T)16 * ei[v + 1] - (T)30 * ei[v + 2] + (T)16 * ei[v + 3] - ei[v + 4]);
+                    }
+                }
+                T qr[VEC], qi[VEC];
+                ldv<T, VEC>(Pg + o, qr);
+                ldv<T, VEC>(Pg + o + blk, qi);
+                v_add<VEC>(ar, qr);
+                v_add<VEC>(ai, qi);
+            }
+        }
+        if (n_nb > 0 || term) {  // 4th-order central d/dp of G
+            T er[VEC + 4], ei[VEC + 4];
+            widen(gr, gi, er, ei);
 #pragma unroll
             for (int v = 0; v < VEC; ++v) {
                 ar[v] += inv12dp * (er[v] - (T)8 * er[v + 1] + (T)8 * er[v + 3] - er[v + 4]);
                 ai[v] += inv12dp * (ei[v] - (T)8 * ei[v + 1] + (T)8 * ei[v + 3] - ei[v + 4]);
             }
         }
-        {  // potential term (with the p-diagonal bath terms) from phase A
+        if constexpr (!PG) {  // potential term (with the p-diagonal bath terms) from phase A
             const int pb = ((rg * RG + r) * S2 + pr) * NP + l0;
 #pragma unroll
             for (int v = 0; v < VEC; ++v) {

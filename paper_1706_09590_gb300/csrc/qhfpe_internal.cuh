@@ -143,10 +143,9 @@ template <typename T, bool MIXED>
 cudaError_t launch_fused(const GridInfo &g, const ElemInfo *elems, const FusedTables<T> &tab, const T *v_in,
                          const T *y, const double *y0, T *v_out, double *y0_out, double h, int mode, int terms,
                          int rep0, int n_rep, cudaStream_t st, const T *Pg = nullptr, int tq = 0, int form = -1);
-// The q-window form of the fused stage kernel (FP32, np 128, one or two states, every term with the
-// potential in the kernel, lanes of one p sign, at most six tier neighbours, linear coupling), unless
+// The q-window form of the fused stage kernel (FP32, np 128, one or two states, every term, lanes of one p sign, at most six tier neighbours, linear coupling), unless
 // QHFPE_FUSED_WINDOW=0; its q rows per block.
-bool fused_window_applies(const GridInfo &g, int terms, bool have_pg);
+bool fused_window_applies(const GridInfo &g, int terms);
 int fused_window_rows(int S);
 int fused_max_rows(int np, int S, int elem_bytes);
 template <typename T>
