@@ -202,6 +202,7 @@ struct Model {
     bool fused = false;         // fused stage kernel available for (np, S)
     double *ftab64 = nullptr;   // its tables (digit-reversed order, np twiddles)
     float *ftab32 = nullptr;
+    float *rtab = nullptr;      // resident propagation: D | L | R | lpp in its transform's order (built on first use)
     FusedTables<double> f64() const
     {
         return {ftab64, ftab64 + tab_n, ftab64 + 2 * tab_n, ftab64 + 3 * tab_n, ftab64 + 3 * tab_n + 2 * np,
@@ -218,6 +219,7 @@ struct Model {
         if (tab64) cudaFree(tab64);
         if (tab32) cudaFree(tab32);
         if (ftab64) cudaFree(ftab64);
+        if (rtab) cudaFree(rtab);
         if (ftab32) cudaFree(ftab32);
         if (tcN) cudaFree(tcN);
         if (tcB) cudaFree(tcB);
@@ -241,6 +243,20 @@ struct Timing {
     }
 };
 
+// Launch shape and device buffers of a resident propagation (qhfpe_resident.cu).
+struct ResidentPlan {
+    int csize = 0, threads = 0, clusters = 0;
+    size_t smem = 0;
+    void *desc = nullptr;   // ResidentMember[n]
+    double *part = nullptr; // trace parts of one launch
+    size_t part_cap = 0;    // doubles
+    ~ResidentPlan()
+    {
+        if (desc) cudaFree(desc);
+        if (part) cudaFree(part);
+    }
+};
+
 // One propagator: a batch of replicas of one model in one arithmetic.
 struct Prop {
     Model *m = nullptr;
@@ -260,6 +276,8 @@ struct Prop {
     void *pdesc = nullptr;      // persistent propagation: this propagator as a one-member batch
     int pdesc_tq = 0;           // its tile height
     unsigned *pbar = nullptr;   // barrier words (count, generation) and the give-up flag
+    int res_state = 0;          // resident propagation: 0 not yet decided, 1 taken, -1 not
+    ResidentPlan res;
 
     void drop_graphs()
     {
@@ -942,10 +960,146 @@ qhfpe_status run_persistent(qhfpe *h, Prop &P, long n_steps, double *trace_dev, 
     return QHFPE_OK;
 }
 
+// ---- resident propagation ------------------------------------------------------------------------
+// Mixed-form two-state propagators with np 32 or 64, linear coupling, no learned closure and the Condon
+// trace, whose lanes' eight p values share a sign.  QHFPE_RESIDENT=0 keeps the launch-per-stage form, as does
+// QHFPE_TILE_ROWS (which pins that form's tile) and kernel timing (which counts its launches).
+bool resident_wanted(const qhfpe *h, const Prop &P)
+{
+    const Model &M = *P.m;
+    if (!P.mixed || P.tc || !M.fused || !resident_supported(P.g.np, P.g.S)) return false;
+    if (M.closure_slot >= 0 || M.noncondon || P.g.c2 != 0.0 || h->persistent || h->timing.enabled) return false;
+    for (int c = 0; c < P.g.np; c += 8)  // (a lane has four or eight)
+        if (((float)(P.g.p_min + c * P.g.dp) < 0.f) != ((float)(P.g.p_min + (c + 7) * P.g.dp) < 0.f)) return false;
+    const char *r = std::getenv("QHFPE_RESIDENT");
+    return !(r && std::strcmp(r, "0") == 0) && !std::getenv("QHFPE_TILE_ROWS");
+}
+
+// Blocks per cluster: the most (up to 16) with which all clusters run at once, so that few replicas spread
+// over many SMs; otherwise the fewest that hold a replica (least halo and barrier work, clusters in
+// waves).  False: a replica does not fit.
+bool resident_plan(const std::vector<const Prop *> &props, ResidentPlan &R)
+{
+    const int np = props[0]->g.np;
+    int nq_max = 1, clusters = 0;
+    for (const Prop *p : props) {
+        nq_max = std::max(nq_max, p->g.nq);
+        clusters += p->g.n_rep;
+    }
+    bool found = false;
+    for (int cs = 16; cs >= 1; cs /= 2) {
+        if (cs > 1 && (nq_max + cs - 1) / cs < 2) continue;
+        size_t smem = 0;
+        int threads = 32;
+        bool fits = true;
+        for (const Prop *p : props) {
+            const int rows = (p->g.nq + cs - 1) / cs;
+            const size_t need = resident_smem(np, p->g.n_elem, rows);
+            fits = fits && need > 0;
+            smem = std::max(smem, need);
+            threads = std::max(threads, resident_threads(np, p->g.n_elem, rows));
+        }
+        if (!fits) continue;
+        int cap = 0;
+        if (resident_capacity(np, cs, threads, smem, &cap) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        if (cap < 1) continue;
+        found = true;
+        R.csize = cs;
+        R.threads = threads;
+        R.smem = smem;
+        R.clusters = clusters;
+        if (cap >= clusters) break;
+    }
+    return found;
+}
+
+qhfpe_status resident_tables(qhfpe *h, Model &M, const double *U)
+{
+    if (M.rtab) return QHFPE_OK;
+    std::vector<double> t;
+    const int np = M.np;
+    build_tables(M, U, t, [np](int pos) { return resident_frequency(np, pos); }, 0, true);
+    std::vector<float> f(t.begin(), t.end());
+    QH_CK(h, dalloc(&M.rtab, f.size()));
+    QH_CK(h, cudaMemcpy(M.rtab, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice));
+    return QHFPE_OK;
+}
+
+// n_steps RK4 steps of every propagator; traces[m] (device, may be nullptr): slots 1..n_steps of each replica.
+qhfpe_status run_resident(qhfpe *h, const std::vector<Prop *> &props, const std::vector<double *> &traces, long stride,
+                          ResidentPlan &R, long n_steps, cudaStream_t st)
+{
+    const int np = props[0]->g.np;
+    std::vector<ResidentMember> d(props.size());
+    const bool record = !traces.empty();
+    if (!R.desc) QH_CK(h, cudaMalloc(&R.desc, d.size() * sizeof(ResidentMember)));
+    const int n_part = R.csize * (R.threads / 32);  // warps of a cluster, each with its part of the trace
+    const size_t per_step = (size_t)R.clusters * n_part * 2;  // doubles of one step's trace parts
+    // steps per launch: bounded so that a launch stays well below a second and the parts below 64 MB
+    const long most = std::max<long>(1, std::min<long>(4096, (8l << 20) / (long)per_step));
+    if (record) {
+        const size_t need = per_step * (size_t)std::min(most, n_steps);
+        if (R.part_cap < need) {
+            if (R.part) cudaFree(R.part);
+            R.part = nullptr;
+            R.part_cap = 0;
+            QH_CK(h, dalloc(&R.part, need));
+            R.part_cap = need;
+        }
+    }
+    for (long done = 0; done < n_steps;) {
+        const int len = (int)std::min(most, n_steps - done);
+        int cluster = 0;
+        size_t part = 0;
+        for (size_t m = 0; m < props.size(); ++m) {
+            const Prop &P = *props[m];
+            ResidentMember &x = d[m];
+            std::memset((void *)&x, 0, sizeof(x));
+            x.g = P.g;
+            x.elems = P.m->elems;
+            x.tab = P.m->rtab;
+            x.tw = P.m->f32().tw;
+            x.sc[0] = stage_scalars<float>(P.g, 0.0);
+            for (int k = 1; k <= 4; ++k) x.sc[k] = stage_scalars<float>(P.g, P.dt / k);
+            x.dt = P.dt;
+            x.y = (float *)P.y;
+            x.lo = (float *)P.vB;
+            x.y0 = P.y0;
+            x.mu = P.m->mu;
+            x.part = record ? R.part + part : nullptr;
+            part += (size_t)P.g.n_rep * len * n_part * 2;
+            x.cluster0 = cluster;
+            cluster += P.g.n_rep;
+            x.rows = (P.g.nq + R.csize - 1) / R.csize;
+        }
+        QH_CK(h, cudaMemcpyAsync(R.desc, d.data(), d.size() * sizeof(ResidentMember), cudaMemcpyHostToDevice, st));
+        QH_CK(h, launch_resident(np, (const ResidentMember *)R.desc, (int)d.size(), R.clusters, R.csize, R.threads, R.smem,
+                                 len, done == 0, st));
+        if (record)
+            for (size_t m = 0; m < props.size(); ++m)
+                QH_CK(h, launch_resident_trace(d[m].part, props[m]->g.n_rep, len, n_part, props[m]->g.dq * props[m]->g.dp,
+                                               traces[m], stride, 1 + done, st));
+        done += len;
+    }
+    return QHFPE_OK;
+}
+
+// The resident form for one propagator, where it applies (decided once per propagator).
+bool resident_ok(qhfpe *h, Prop &P)
+{
+    if (!resident_wanted(h, P)) return false;
+    if (P.res_state == 0) P.res_state = resident_plan({&P}, P.res) ? 1 : -1;
+    return P.res_state > 0;
+}
+
 qhfpe_status run_steps(qhfpe *h, Prop &P, long n_steps, double *trace_dev, long stride)
 {
     cudaStream_t st = h->stream;
-    if (!P.tq && P.m->fused && n_steps > 0) {
+    const bool resident = n_steps > 0 && resident_ok(h, P);
+    if (!resident && !P.tq && P.m->fused && n_steps > 0) {
         qhfpe_status r = autotune(h, P);
         if (r != QHFPE_OK) return r;
     }
@@ -955,6 +1109,12 @@ qhfpe_status run_steps(qhfpe *h, Prop &P, long n_steps, double *trace_dev, long 
         QH_CK(h, cudaGetLastError());
         if (P.mixed) QH_CK(h, launch_trace<double>(P.g, P.y0, P.g.tier0_rep_stride, P.m->mu, P.sink, 1, P.partial, st, P.m->trace_mu_q()));
         else QH_CK(h, launch_trace<double>(P.g, (const double *)P.y, P.g.rep_stride, P.m->mu, P.sink, 1, P.partial, st, P.m->trace_mu_q()));
+    }
+    if (resident) {
+        qhfpe_status r = resident_tables(h, *P.m, h->U.data());
+        if (r != QHFPE_OK) return r;
+        return run_resident(h, {&P}, record ? std::vector<double *>{trace_dev} : std::vector<double *>{}, stride, P.res,
+                            n_steps, st);
     }
     if (n_steps > 0 && persistent_ok(h, P)) return run_persistent(h, P, n_steps, trace_dev, stride);
     if (h->timing.enabled) {
@@ -2193,6 +2353,8 @@ struct qhfpe_batch {
     void *pdesc = nullptr;      // persistent propagation: this propagator as a one-member batch
     int pdesc_tq = 0;           // its tile height
     unsigned *pbar = nullptr;   // barrier words (count, generation) and the give-up flag
+    int res_state = 0;          // resident propagation: 0 not yet decided, 1 taken, -1 not
+    ResidentPlan res;
     ~qhfpe_batch()
     {
         for (auto &a : graphs)
@@ -2368,7 +2530,17 @@ qhfpe_status qhfpe_batch_step(qhfpe_batch_t *b, long n_steps, double *const *tra
     // every member's earlier work (on its own stream) is complete before the batch touches its buffers
     for (qhfpe *h : b->mem) QH_CK(h, cudaStreamSynchronize(h->stream));
     cudaStream_t st = h0->stream;
-    if (!b->tq && n_steps > 0 && (r = batch_autotune(b, st)) != QHFPE_OK) return r;
+    bool resident = n_steps > 0;
+    for (qhfpe *h : b->mem) resident = resident && resident_wanted(h, *h->main);
+    if (resident) {
+        if (b->res_state == 0) {
+            std::vector<const Prop *> props;
+            for (qhfpe *h : b->mem) props.push_back(h->main.get());
+            b->res_state = resident_plan(props, b->res) ? 1 : -1;
+        }
+        resident = b->res_state > 0;
+    }
+    if (!resident && !b->tq && n_steps > 0 && (r = batch_autotune(b, st)) != QHFPE_OK) return r;
     const bool record = trace_out != nullptr;
     const long stride = n_steps + 1;
     if (record)
@@ -2385,6 +2557,17 @@ qhfpe_status qhfpe_batch_step(qhfpe_batch_t *b, long n_steps, double *const *tra
                                               st, P.m->trace_mu_q()));
         }
     long done = 0;
+    if (resident) {
+        std::vector<Prop *> props;
+        std::vector<double *> traces;
+        for (qhfpe *h : b->mem) {
+            if ((r = resident_tables(h, *h->model, h->U.data())) != QHFPE_OK) return r;
+            props.push_back(h->main.get());
+            if (record) traces.push_back(h->main->trace_buf);
+        }
+        if ((r = run_resident(h0, props, traces, stride, b->res, n_steps, st)) != QHFPE_OK) return r;
+        done = n_steps;
+    }
     while (done < n_steps) {
         const int chunk = (n_steps - done >= kGraphChunk) ? 1 : 0;
         const int len = chunk ? kGraphChunk : 1;

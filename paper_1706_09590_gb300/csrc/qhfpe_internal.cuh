@@ -196,6 +196,35 @@ cudaError_t launch_barrier_selftest(unsigned *bar_words, int *err, unsigned long
                                     cudaStream_t st);
 int trace_chunks(int n_rep, size_t blk);
 
+// ---- cluster-resident propagation (qhfpe_resident.cu) -----------------------------------------------------
+// One propagator of a resident launch: replica r is cluster cluster0 + r, block c of the cluster owns the q
+// rows c * rows .. of every element.
+struct ResidentMember {
+    GridInfo g;
+    const ElemInfo *elems;
+    const float *tab;         // D | L | R [S][S][nq][np] and lpp [np] in the resident transform's order
+    const float *tw;          // np twiddles
+    StageScalars<float> sc[5];  // [k]: stage k = 1..4 (h = dt / k)
+    double dt;
+    float *y, *lo;            // FP32 state; low halves of its FP64 zeroth tier, same layout
+    double *y0;
+    const double *mu;
+    double *part;             // trace parts [n_rep][n_steps][warps of a cluster] complex, or nullptr
+    int cluster0;
+    int rows;
+};
+bool resident_supported(int np, int S);
+int resident_frequency(int np, int pos);  // frequency at each position of its transform
+size_t resident_smem(int np, int n_elem, int rows);  // 0: a block cannot have that much
+int resident_threads(int np, int n_elem, int rows);
+// clusters of csize blocks that fit on the device at once (0: that size cannot run)
+cudaError_t resident_capacity(int np, int csize, int threads, size_t smem, int *clusters);
+// n_steps RK4 steps of every member (device array, cluster0 ascending from 0); first: (re)compute lo
+cudaError_t launch_resident(int np, const ResidentMember *members, int n_mem, int clusters, int csize, int threads,
+                            size_t smem, int n_steps, bool first, cudaStream_t st);
+cudaError_t launch_resident_trace(const double *part, int n_rep, int n_steps, int n_part, double scale, double *out,
+                                  long stride, long slot0, cudaStream_t st);
+
 // ---- tensor-core potential term (qhfpe_tc.cu) ----------------------------------------------------------
 bool tc_supported(int np, int S);
 cudaError_t prepare_tc(int np, int S);
