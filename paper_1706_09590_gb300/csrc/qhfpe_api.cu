@@ -202,6 +202,7 @@ struct Model {
     bool fused = false;         // fused stage kernel available for (np, S)
     double *ftab64 = nullptr;   // its tables (digit-reversed order, np twiddles)
     float *ftab32 = nullptr;
+    int tuned_tq = 0, tuned_form = -1;  // ground model: the tile that the first equilibration chose
     float *rtab = nullptr;      // resident propagation: D | L | R | lpp in its transform's order (built on first use)
     FusedTables<double> f64() const
     {
@@ -829,27 +830,37 @@ qhfpe_status autotune(qhfpe *h, Prop &P)
     cudaEvent_t a, b;
     QH_CK(h, cudaEventCreate(&a));
     QH_CK(h, cudaEventCreate(&b));
-    // one right-hand side of every replica into vB with the given form and tile, timed over three launches
+    float best = 1e30f, ms = 0.f;
+    // right-hand sides of every replica into vB with the given form and tile: one to warm up, one timed, and two
+    // more unless that one was far behind the best so far; *ms for three
     auto time_one = [&](int form, int tq, float *ms) -> qhfpe_status {
-        for (int rep = 0; rep < 4; ++rep) {
-            if (rep == 1) QH_CK(h, cudaEventRecord(a, st));
-            cudaError_t e;
-            if (P.mixed)
-                e = launch_fused<float, true>(P.g, M.elems, M.f32(), (const float *)P.y, (const float *)P.y, P.y0,
-                                              (float *)P.vB, nullptr, 0.0, 0, QHFPE_TERM_ALL, 0, P.g.n_rep, st,
-                                              P.tc ? (const float *)P.P : nullptr, tq, form);
-            else
-                e = launch_fused<double, false>(P.g, M.elems, M.f64(), (const double *)P.y, (const double *)P.y,
-                                                nullptr, (double *)P.vB, nullptr, 0.0, 0, QHFPE_TERM_ALL, 0, P.g.n_rep,
-                                                st, nullptr, tq, form);
-            QH_CK(h, e);
+        *ms = 0.f;
+        for (int n : {1, 2}) {
+            for (int rep = n - 2; rep < n; ++rep) {  // (n = 1: launch -1 is the warm-up)
+                if (rep == 0) QH_CK(h, cudaEventRecord(a, st));
+                cudaError_t e;
+                if (P.mixed)
+                    e = launch_fused<float, true>(P.g, M.elems, M.f32(), (const float *)P.y, (const float *)P.y, P.y0,
+                                                  (float *)P.vB, nullptr, 0.0, 0, QHFPE_TERM_ALL, 0, P.g.n_rep, st,
+                                                  P.tc ? (const float *)P.P : nullptr, tq, form);
+                else
+                    e = launch_fused<double, false>(P.g, M.elems, M.f64(), (const double *)P.y, (const double *)P.y,
+                                                    nullptr, (double *)P.vB, nullptr, 0.0, 0, QHFPE_TERM_ALL, 0, P.g.n_rep,
+                                                    st, nullptr, tq, form);
+                QH_CK(h, e);
+            }
+            float t = 0.f;
+            QH_CK(h, cudaEventRecord(b, st));
+            QH_CK(h, cudaEventSynchronize(b));
+            QH_CK(h, cudaEventElapsedTime(&t, a, b));
+            *ms += t;
+            if (n == 1 && 3.f * t > 1.25f * best) {
+                *ms = 3.f * t;
+                break;
+            }
         }
-        QH_CK(h, cudaEventRecord(b, st));
-        QH_CK(h, cudaEventSynchronize(b));
-        QH_CK(h, cudaEventElapsedTime(ms, a, b));
         return QHFPE_OK;
     };
-    float best = 1e30f, ms = 0.f;
     int best_tq = 1, best_form = 0;
     // the kernel form: the q-window kernel (fixed tile) where it applies, against the general kernel
     if (P.mixed && fused_window_applies(P.g, QHFPE_TERM_ALL)) {
@@ -861,9 +872,13 @@ qhfpe_status autotune(qhfpe *h, Prop &P)
     }
     // tile heights of the general kernel, between the powers of two as well: the block count (tiles x
     // elements x replicas) against the blocks resident at once decides how full the last wave is
-    static const int cand[] = {1, 2, 3, 4, 5, 6, 8, 12, 16};
-    for (int tq : cand) {
-        if (tq > tmax) break;
+    const int first = std::min(fused_rows_per_tile(P.g.np, P.g.S, esize), tmax);  // a good one, to leave bad ones early
+    bool timed[17] = {};
+    for (int c : {first, 1, 2, 3, 4, 5, 6, 8, 12, 16}) {
+        if (c > tmax) break;
+        const int tiles = (P.g.nq + c - 1) / c, tq = (P.g.nq + tiles - 1) / tiles;  // as many tiles, of one height
+        if (timed[tq]) continue;
+        timed[tq] = true;
         qhfpe_status r = time_one(0, tq, &ms);
         if (r != QHFPE_OK) return r;
         if (ms < best) {
@@ -1837,9 +1852,13 @@ qhfpe_status equilibrium_start(qhfpe_t *h, std::unique_ptr<Prop> &GP)
     Model &G = *h->ground;
     r = make_prop(h, &G, 1, false, p.dt, GP);
     if (r != QHFPE_OK) return r;
+    if (!std::getenv("QHFPE_TILE_ROWS")) {
+        GP->tq = G.tuned_tq;
+        GP->form = G.tuned_form;
+    }
     const size_t blk = (size_t)nq * np;
     const size_t gn = (size_t)G.n_elem * blk;
-    std::vector<double> w0(2 * gn, 0.0);
+    std::vector<double> w0(2 * blk, 0.0);  // the zeroth element; the others start from zero
     double norm = 0.0;
     const double dq = (p.q_max - p.q_min) / nq, dp = (p.p_max - p.p_min) / np;
     for (int i = 0; i < nq; ++i)
@@ -1852,9 +1871,10 @@ qhfpe_status equilibrium_start(qhfpe_t *h, std::unique_ptr<Prop> &GP)
     norm *= dq * dp;
     for (size_t c = 0; c < blk; ++c) w0[2 * c] /= norm;
     const size_t full = (size_t)G.n_elem * S * S * blk;
-    r = ensure_scratch(h, std::max(gn, full) * 2 * sizeof(double) + 64);
+    r = ensure_scratch(h, std::max(gn, full) * 2 * sizeof(double) + QH_NORM_DOUBLES * sizeof(double));
     if (r != QHFPE_OK) return r;
-    QH_CK(h, cudaMemcpyAsync(h->scratch, w0.data(), gn * 2 * sizeof(double), cudaMemcpyHostToDevice, st));
+    QH_CK(h, cudaMemsetAsync(h->scratch, 0, gn * 2 * sizeof(double), st));
+    QH_CK(h, cudaMemcpyAsync(h->scratch, w0.data(), w0.size() * sizeof(double), cudaMemcpyHostToDevice, st));
     return set_from_canonical(h, *GP, h->scratch, 0, 1);
 }
 
@@ -1876,8 +1896,7 @@ qhfpe_status equilibrium_residual(qhfpe_t *h, Prop &GP, double *res)
                                               QHFPE_TERM_ALL, 0, 1, st)));
     }
     const size_t real = (size_t)G.n_elem * GP.g.elem_stride;
-    QH_CK(h, launch_norm2((const double *)GP.vA, real, h->scratch, st));
-    QH_CK(h, launch_norm2((const double *)GP.y, real, h->scratch + 1, st));
+    QH_CK(h, launch_norm2((const double *)GP.vA, (const double *)GP.y, real, h->scratch, st));
     double nn[2];
     QH_CK(h, cudaMemcpyAsync(nn, h->scratch, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
     QH_CK(h, cudaStreamSynchronize(st));
@@ -1890,6 +1909,8 @@ qhfpe_status equilibrium_residual(qhfpe_t *h, Prop &GP, double *res)
 // also written to every replica.
 qhfpe_status equilibrium_embed(qhfpe_t *h, Prop &GP)
 {
+    h->ground->tuned_tq = GP.tq;
+    h->ground->tuned_form = GP.form;
     const int S = h->p.n_states;
     const Model &G = *h->ground;
     const size_t blk = (size_t)h->p.nq * h->p.np;

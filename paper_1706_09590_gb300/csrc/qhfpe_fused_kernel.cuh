@@ -641,7 +641,7 @@ template <int NP, int S> __device__ __forceinline__ void potential_to_double(dou
     }
 }
 
-// A tier coupling's weight for the fixed-point sums: w = c 2^(k - 62), |c| in [2^61, 2^62).
+// A factor for fixed-point products: w = c 2^(k - 62), |c| in [2^61, 2^62).
 struct FixedWeight {
     qhfx::Half c;
     int k;
@@ -653,7 +653,6 @@ __device__ __forceinline__ FixedWeight fixed_weight(double w)
     const long long m = qhfx::to_fixed<62>(w, ex);
     return FixedWeight{qhfx::halves(m), ex - 1022};
 }
-constexpr int FIXED_MAXNB = 12;  // terms of a tier sum: 12 x 18 x 2^55 stays below 2^63
 
 // Phase B of the FP64 form (linear coupling, all terms, the potential and the p-diagonal bath terms already
 // in X): kinetic term, tier couplings and update of the block's rows.  As in the transforms
@@ -662,23 +661,23 @@ constexpr int FIXED_MAXNB = 12;  // terms of a tier sum: 12 x 18 x 2^55 stays be
 //            pair; for each of its p columns the nine rows read are brought to the column's largest exponent
 //            (62 bits below it) once, and the four sums of six are exact.  Where the rows' own exponents are
 //            more than eight apart each of the four takes its own.
-//   tiers    G = sum of the neighbours' rows, weighted; every term (value times weight) is brought to the row's
-//            largest exponent, 55 bits below it, and the p difference of G (weights 1, 8) is exact.
+//   tiers    G = sum of the neighbours' rows, weighted, in FP64 (one instruction per value and neighbour, on a
+//            pipe that has room for them; in integers the conversions alone took twenty); its row is brought
+//            to the largest exponent, 57 bits below it, and the p difference (weights 1, 8) is exact.
 // Quantising at 2^-54 to 2^-62 of the largest term is below the rounding of the FP64 sums, whose partial sums of
-// up to 100 times the values round at 2^-53.  Three FP64 instructions per value remain (the scaled p difference,
-// p W^(n-e_0), out = y + h L) of 43.
+// up to 100 times the values round at 2^-53.
 // Infinities, NaN and values from 2^1007: a column or row that holds one gives NaN.
 template <int NP, int S>
 __device__ __forceinline__ void
 rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__restrict__ v_in, const double *y, double *v_out,
-           int mode, size_t ebase, int i0, int rows, const long long *nb_off, const FixedWeight *nb_fw, const double *nb_wa,
+           int mode, size_t ebase, int i0, int rows, const long long *nb_off, const double *nb_wg, const double *nb_wa,
            int n_up, int n_d0, int n_nb, bool term, double2 *X, const double *pgrid)
 {
     using namespace qhfx;
     constexpr int S2 = S * S;
     constexpr int VEC = NP / 32;              // a warp holds a p row
-    constexpr int RG = 4;                     // q rows per unit
-    constexpr int BITS = 55;
+    constexpr int RG = 4;                     // q rows per unit, at most
+    constexpr int BITS = 57;                  // of G below its row's largest value: 18 x 2^57 stays below 2^62
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t blk = g.blk;
     const int nq = g.nq;
@@ -692,10 +691,11 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
     }
     const int first = neg ? -2 : -3;
     const double bad = bitsd(0x7ff8000000000000ull);
+    const int rg = min(RG, (rows * S2 + FTHREADS / 32 - 1) / (FTHREADS / 32));  // fewer where warps would idle
 #pragma unroll 1
-    for (int u = warp; u < ((rows + RG - 1) / RG) * S2; u += FTHREADS / 32) {
-        const int pr = u % S2, r0 = (u / S2) * RG;
-        const int nr = min(RG, rows - r0);
+    for (int u = warp; u < ((rows + rg - 1) / rg) * S2; u += FTHREADS / 32) {
+        const int pr = u % S2, r0 = (u / S2) * rg;
+        const int nr = min(rg, rows - r0);
         const int ia = i0 + r0;
         const size_t poff = ebase + (size_t)pr * 2 * blk;
 #pragma unroll 1
@@ -759,18 +759,15 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                     for (int r = 0; r < RG; ++r)
                         if (r < nr) emit(r, x + r, E);
                 } else {  // steep in q: an exponent for each row
-#pragma unroll 1
-                    for (int r = 0; r < nr; ++r) {
-                        Half x[6];
-                        double w[6];
+#pragma unroll
+                    for (int r = 0; r < RG; ++r) {
+                        if (r >= nr) continue;
                         int er = EXP_MIN;
 #pragma unroll
-                        for (int t = 0; t < 6; ++t) {
-                            w[t] = value(r + t);
-                            er = max(er, exponent_of(w[t]));
-                        }
+                        for (int t = 0; t < 6; ++t) er = max(er, ex[r + t]);
+                        Half x[6];
 #pragma unroll
-                        for (int t = 0; t < 6; ++t) x[t] = halves(to_fixed<62>(w[t], er));
+                        for (int t = 0; t < 6; ++t) x[t] = halves(to_fixed<62>(raw[r + t], er));
                         emit(r, x, er);
                     }
                 }
@@ -789,72 +786,60 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                 double a[VEC];
 #pragma unroll
                 for (int v = 0; v < VEC; ++v) a[v] = Xat(r, v);  // potential and kinetic terms
-                // G at the row's exponent E, built up term by term
-                long long G[VEC];
-                int E = EXP_MIN;
+                // tier couplings: G = sum of the neighbours, weighted, in FP64
+                double G[VEC];
 #pragma unroll
-                for (int v = 0; v < VEC; ++v) G[v] = 0;
-                // the neighbours in turn, the next one's values in flight; last the terminator's r_0 p W
-                const int n_terms = n_nb + (term ? 1 : 0);
-                const auto source = [&](int n) { return v_in + (long long)o + (n < n_nb ? nb_off[n] : 0); };
-                double next[VEC];
-                if (n_terms > 0) ldv<double, VEC>(source(0), next);
+                for (int v = 0; v < VEC; ++v) G[v] = 0.0;
+                {
+                    double next[VEC];
+                    if (n_nb > 0) ldv<double, VEC>(v_in + (long long)o + nb_off[0], next);
 #pragma unroll 1
-                for (int n = 0; n < n_terms; ++n) {
-                    double w[VEC];
+                    for (int n = 0; n < n_nb; ++n) {
+                        double w[VEC];
+                        const double wg = nb_wg[n];
 #pragma unroll
-                    for (int v = 0; v < VEC; ++v) w[v] = next[v];
-                    if (n + 1 < n_terms) ldv<double, VEC>(source(n + 1), next);
-                    if (n >= n_d0) {  // warp-uniform; (the barrier keeps it a branch: FP64 instructions that
-                                      // are only predicated off take their 64 clocks all the same)
-                        __syncwarp();
-                        if (n >= n_nb) {
+                        for (int v = 0; v < VEC; ++v) w[v] = next[v];
+                        if (n + 1 < n_nb) ldv<double, VEC>(v_in + (long long)o + nb_off[n + 1], next);
 #pragma unroll
-                            for (int v = 0; v < VEC; ++v) w[v] *= sc.r0 * p[v];
-                        } else {
+                        for (int v = 0; v < VEC; ++v) G[v] = fma(wg, w[v], G[v]);
+                        if (n >= n_d0) {  // warp-uniform; (the barrier keeps it a branch: FP64 instructions that
+                                          // are only predicated off take their 64 clocks all the same)
+                            __syncwarp();
                             const double wa = nb_wa[n];
 #pragma unroll
                             for (int v = 0; v < VEC; ++v) a[v] = fma(n == n_d0 ? pw[v] : p[v] * wa, w[v], a[v]);
                         }
                     }
-                    const bool weighted = n >= n_up && n < n_nb;
-                    const FixedWeight fw = nb_fw[n < FIXED_MAXNB ? n : 0];
-                    const int k = weighted ? fw.k : 0;
-                    int em = 0;
+                }
+                if (term) {  // r_0 p W of the Eq. (GMFP) terminator
+                    __syncwarp();
+                    double w[VEC];
+                    ldv<double, VEC>(v_in + o, w);
 #pragma unroll
-                    for (int v = 0; v < VEC; ++v) em = max(em, exponent_of(w[v]));
-                    em = em >= EXP_BIG ? 2 * EXP_BIG : em + k;
-                    em = __reduce_max_sync(0xffffffffu, em);
-                    if (em > E) {  // warp-uniform
-#pragma unroll
-                        for (int v = 0; v < VEC; ++v) G[v] = shr_s(G[v], em - E);
-                        E = em;
-                    }
-#pragma unroll
-                    for (int v = 0; v < VEC; ++v) {
-                        const long long x = to_fixed<BITS + 2>(w[v], E - k);
-                        if (weighted) {
-                            G[v] += mul_hi(halves(x), fw.c);
-                        } else {
-                            G[v] += x >> 2;
-                        }
-                    }
+                    for (int v = 0; v < VEC; ++v) G[v] = fma(sc.r0 * p[v], w[v], G[v]);
                 }
                 if (n_nb > 0 || term) {  // 4th-order central d/dp of G, periodic p, neighbours through the warp
+                    int E = EXP_MIN;
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) E = max(E, exponent_of(G[v]));
+                    E = __reduce_max_sync(0xffffffffu, E);
+                    long long Gi[VEC];
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) Gi[v] = to_fixed<BITS>(G[v], E);
                     long long e[VEC + 4];
 #pragma unroll
-                    for (int v = 0; v < VEC; ++v) e[v + 2] = G[v];
+                    for (int v = 0; v < VEC; ++v) e[v + 2] = Gi[v];
                     const unsigned all = 0xffffffffu;
                     if constexpr (VEC == 1) {
-                        e[0] = __shfl_sync(all, G[0], (lane + 30) & 31);
-                        e[1] = __shfl_sync(all, G[0], (lane + 31) & 31);
-                        e[3] = __shfl_sync(all, G[0], (lane + 1) & 31);
-                        e[4] = __shfl_sync(all, G[0], (lane + 2) & 31);
+                        e[0] = __shfl_sync(all, Gi[0], (lane + 30) & 31);
+                        e[1] = __shfl_sync(all, Gi[0], (lane + 31) & 31);
+                        e[3] = __shfl_sync(all, Gi[0], (lane + 1) & 31);
+                        e[4] = __shfl_sync(all, Gi[0], (lane + 2) & 31);
                     } else {
-                        e[0] = __shfl_sync(all, G[VEC - 2], (lane + 31) & 31);
-                        e[1] = __shfl_sync(all, G[VEC - 1], (lane + 31) & 31);
-                        e[VEC + 2] = __shfl_sync(all, G[0], (lane + 1) & 31);
-                        e[VEC + 3] = __shfl_sync(all, G[1], (lane + 1) & 31);
+                        e[0] = __shfl_sync(all, Gi[VEC - 2], (lane + 31) & 31);
+                        e[1] = __shfl_sync(all, Gi[VEC - 1], (lane + 31) & 31);
+                        e[VEC + 2] = __shfl_sync(all, Gi[0], (lane + 1) & 31);
+                        e[VEC + 3] = __shfl_sync(all, Gi[1], (lane + 1) & 31);
                     }
 #pragma unroll
                     for (int v = 0; v < VEC; ++v) {
@@ -952,7 +937,6 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
 
     __shared__ long long nb_off[3 * QH_MAX_MODES];
     __shared__ T nb_wg[3 * QH_MAX_MODES], nb_wa[3 * QH_MAX_MODES];
-    __shared__ FixedWeight nb_fw[FIXED_MAXNB];  // FP64 form: nb_wg for the fixed-point sums
     __shared__ long long mx_off[QH_MAX_MODES];  // nonlinear coupling: mixed-derivative neighbours
     __shared__ T mx_w[QH_MAX_MODES];
     __shared__ int s_nmx;
@@ -997,21 +981,6 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
         s_cnt[2] = n;
         s_cnt[3] = (terms & 8) && E.terminator;
         s_ngam = (terms & 4) ? (T)E.ngam : (T)0;
-    }
-    if constexpr (sizeof(T) == sizeof(double) && !NL) {
-        // (read after the barriers of phase A)
-        if (threadIdx.x >= 32 && threadIdx.x < 32 + FIXED_MAXNB) {
-            const ElemInfo &E = elems[e];
-            const int a = threadIdx.x - 32;
-            // the order of nb_wg: up, down without a p term, down with one
-            int n = E.n_up;
-            for (int pass = 0; pass < 2; ++pass)
-                for (int d = 0; d < E.n_dn; ++d)
-                    if ((E.wr[d] != 0.0) == (pass == 1)) {
-                        if (n == a) nb_fw[a] = fixed_weight(E.wc[d]);
-                        ++n;
-                    }
-        }
     }
     if (!warm)
         for (int t = threadIdx.x; t < NP; t += FTHREADS) {
@@ -1080,8 +1049,8 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
     if constexpr (sizeof(T) == sizeof(double) && !NL) {
         // the fixed-point form: all terms, the potential in X, every lane's p values of one sign
         const bool one_sign = __all_sync(0xffffffffu, (pgrid[lane * (NP / 32)] < (T)0) == (pgrid[lane * (NP / 32) + NP / 32 - 1] < (T)0));
-        if (fold && terms == QHFPE_TERM_ALL && one_sign && n_nb + (term ? 1 : 0) <= FIXED_MAXNB) {
-            rows_fixed<NP, S>(g, sc, v_in, y, v_out, mode, ebase, i0, rows, nb_off, nb_fw, nb_wa, n_up, n_d0, n_nb, term, X,
+        if (fold && terms == QHFPE_TERM_ALL && one_sign) {
+            rows_fixed<NP, S>(g, sc, v_in, y, v_out, mode, ebase, i0, rows, nb_off, nb_wg, nb_wa, n_up, n_d0, n_nb, term, X,
                               pgrid);
             return;
         }

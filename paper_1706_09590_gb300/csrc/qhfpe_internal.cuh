@@ -291,7 +291,9 @@ cudaError_t launch_complex_combine(const double *a, const double *b, double ar, 
                                    double *out, size_t n, cudaStream_t st);
 cudaError_t launch_first_order_combine(int S, size_t blk, int n_elem, int n_omega, const double *mu,
                                        const double *acc_c, const double *acc_s, double *out, cudaStream_t st);
-cudaError_t launch_norm2(const double *x, size_t n, double *out_dev, cudaStream_t st);
+// squared 2-norms of x and y into out_dev[0], out_dev[1]; out_dev holds QH_NORM_DOUBLES doubles
+#define QH_NORM_DOUBLES (2 + 2 * 152)
+cudaError_t launch_norm2(const double *x, const double *y, size_t n, double *out_dev, cudaStream_t st);
 // DFMA throughput probe: blocks x 256 threads, each n_iter x 64 DFMAs; out: blocks * 256 doubles
 cudaError_t launch_dfma_rate(int blocks, int n_iter, double *out, cudaStream_t st);
 cudaError_t launch_wait_flag(const int *flag, unsigned long long limit_ns, int *status, cudaStream_t st);
