@@ -307,6 +307,54 @@ __device__ __forceinline__ void stv(T *p, const T *in)
     }
 }
 
+// The same for rows of the state in global memory: 32-byte accesses where a lane has that much (FP32 np 256, FP64
+// np >= 128; rows are 32-byte aligned there).  Two 16-byte accesses of stride 32 touch every sector twice: np 256
+// with three states spent two thirds of its L1 wavefronts on them.  256 x 256, depth 10, three states: 8.60 -> 7.78
+// ms a step; 96 x 128, depth 8 in FP64: 1 %.
+template <typename T, int VEC>
+__device__ __forceinline__ void ldrow(const T *p, T *o)
+{
+    if constexpr (VEC * sizeof(T) % 32 == 0) {
+        constexpr int N = 32 / (int)sizeof(T);
+#pragma unroll
+        for (int c = 0; c < VEC; c += N) {
+            const size_t a = __cvta_generic_to_global(p + c);
+            if constexpr (sizeof(T) == 4)
+                asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                             : "=f"(o[c]), "=f"(o[c + 1]), "=f"(o[c + 2]), "=f"(o[c + 3]), "=f"(o[c + 4]), "=f"(o[c + 5]),
+                               "=f"(o[c + 6]), "=f"(o[c + 7])
+                             : "l"(a));
+            else
+                asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                             : "=d"(o[c]), "=d"(o[c + 1]), "=d"(o[c + 2]), "=d"(o[c + 3])
+                             : "l"(a));
+        }
+    } else {
+        ldv<T, VEC>(p, o);
+    }
+}
+template <typename T, int VEC>
+__device__ __forceinline__ void strow(T *p, const T *i)
+{
+    if constexpr (VEC * sizeof(T) % 32 == 0) {
+        constexpr int N = 32 / (int)sizeof(T);
+#pragma unroll
+        for (int c = 0; c < VEC; c += N) {
+            const size_t a = __cvta_generic_to_global(p + c);
+            if constexpr (sizeof(T) == 4)
+                asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(a), "f"(i[c]), "f"(i[c + 1]),
+                             "f"(i[c + 2]), "f"(i[c + 3]), "f"(i[c + 4]), "f"(i[c + 5]), "f"(i[c + 6]), "f"(i[c + 7])
+                             : "memory");
+            else
+                asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(a), "d"(i[c]), "d"(i[c + 1]), "d"(i[c + 2]),
+                             "d"(i[c + 3])
+                             : "memory");
+        }
+    } else {
+        stv<T, VEC>(p, i);
+    }
+}
+
 // 128-thread blocks (measured faster than 256: more independent blocks per SM keep phase A and phase B
 // of different blocks overlapping, and each barrier stalls four warps).  The kernel waits mostly on L2
 // loads, so resident warps count: FP32 with one or two states runs seven blocks per SM (72 registers;
@@ -433,8 +481,8 @@ __device__ __forceinline__ void fill_fixed(double2 *X, const double *__restrict_
         const int pr = act ? rp % S2 : 0, r = act ? rp / S2 : 0;
         const double *src = v + (size_t)pr * 2 * blk + (size_t)(i0 + r) * NP + l;
         double re[LV], im[LV];
-        ldv<double, LV>(src, re);
-        ldv<double, LV>(src + blk, im);
+        ldrow<double, LV>(src, re);
+        ldrow<double, LV>(src + blk, im);
         int E = common_exponent<LV>(re, im);
 #pragma unroll
         for (int o = PL / 2; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
@@ -792,14 +840,14 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                 for (int v = 0; v < VEC; ++v) G[v] = 0.0;
                 {
                     double next[VEC];
-                    if (n_nb > 0) ldv<double, VEC>(v_in + (long long)o + nb_off[0], next);
+                    if (n_nb > 0) ldrow<double, VEC>(v_in + (long long)o + nb_off[0], next);
 #pragma unroll 1
                     for (int n = 0; n < n_nb; ++n) {
                         double w[VEC];
                         const double wg = nb_wg[n];
 #pragma unroll
                         for (int v = 0; v < VEC; ++v) w[v] = next[v];
-                        if (n + 1 < n_nb) ldv<double, VEC>(v_in + (long long)o + nb_off[n + 1], next);
+                        if (n + 1 < n_nb) ldrow<double, VEC>(v_in + (long long)o + nb_off[n + 1], next);
 #pragma unroll
                         for (int v = 0; v < VEC; ++v) G[v] = fma(wg, w[v], G[v]);
                         if (n >= n_d0) {  // warp-uniform; (the barrier keeps it a branch: FP64 instructions that
@@ -814,7 +862,7 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                 if (term) {  // r_0 p W of the Eq. (GMFP) terminator
                     __syncwarp();
                     double w[VEC];
-                    ldv<double, VEC>(v_in + o, w);
+                    ldrow<double, VEC>(v_in + o, w);
 #pragma unroll
                     for (int v = 0; v < VEC; ++v) G[v] = fma(sc.r0 * p[v], w[v], G[v]);
                 }
@@ -851,11 +899,11 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                 }
                 if (mode != 0) {
                     double b[VEC];
-                    ldv<double, VEC>(y + o, b);
+                    ldrow<double, VEC>(y + o, b);
 #pragma unroll
                     for (int v = 0; v < VEC; ++v) a[v] = fma(sc.h, a[v], b[v]);
                 }
-                stv<double, VEC>(v_out + o, a);
+                strow<double, VEC>(v_out + o, a);
             }
         }
     }
@@ -1106,8 +1154,8 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
 #pragma unroll
                 for (int b = 0; b < 3; ++b) {
                     if (interior) {
-                        ldv<T, VEC>(rre + (t0 + b) * NP, sr[b]);
-                        ldv<T, VEC>(rim + (t0 + b) * NP, si[b]);
+                        ldrow<T, VEC>(rre + (t0 + b) * NP, sr[b]);
+                        ldrow<T, VEC>(rim + (t0 + b) * NP, si[b]);
                         continue;
                     }
                     int ii = i + t0 + b - 3 + sh;
@@ -1117,8 +1165,8 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
                         ok = true;
                     }
                     if (ok) {
-                        ldv<T, VEC>(Vre + (size_t)ii * NP + l0, sr[b]);
-                        ldv<T, VEC>(Vim + (size_t)ii * NP + l0, si[b]);
+                        ldrow<T, VEC>(Vre + (size_t)ii * NP + l0, sr[b]);
+                        ldrow<T, VEC>(Vim + (size_t)ii * NP + l0, si[b]);
                     } else {
 #pragma unroll
                         for (int v = 0; v < VEC; ++v) sr[b][v] = si[b][v] = (T)0;
@@ -1157,8 +1205,8 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
                         ii = ii < 0 ? ii + nq : ii - nq;
                     }
                     T rr[VEC], ri[VEC];
-                    ldv<T, VEC>(Vre + (size_t)ii * NP + l0, rr);
-                    ldv<T, VEC>(Vim + (size_t)ii * NP + l0, ri);
+                    ldrow<T, VEC>(Vre + (size_t)ii * NP + l0, rr);
+                    ldrow<T, VEC>(Vim + (size_t)ii * NP + l0, ri);
 #pragma unroll
                     for (int v = 0; v < VEC; ++v) {
                         const T c = pcol[v] < (T)0 ? cneg[d + 3] : cpos[d + 3];
@@ -1169,8 +1217,8 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
                 v_fma<VEC>(ar, pk, kr);
                 v_fma<VEC>(ai, pk, ki);
             }
-            ldv<T, VEC>(Vre + (size_t)i * NP + l0, wr);
-            ldv<T, VEC>(Vim + (size_t)i * NP + l0, wi);
+            ldrow<T, VEC>(Vre + (size_t)i * NP + l0, wr);
+            ldrow<T, VEC>(Vim + (size_t)i * NP + l0, wi);
         }
         if (ngam != (T)0) {
             v_axpy<VEC>(ar, -ngam, wr);
@@ -1183,16 +1231,16 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
         for (int a = 0; a < n_up; ++a) {
             const T *u = v_in + (long long)o + nb_off[a];
             T xr[VEC], xi[VEC];
-            ldv<T, VEC>(u, xr);
-            ldv<T, VEC>(u + blk, xi);
+            ldrow<T, VEC>(u, xr);
+            ldrow<T, VEC>(u + blk, xi);
             v_add<VEC>(gr, xr);
             v_add<VEC>(gi, xi);
         }
         for (int a = n_up; a < n_d0; ++a) {
             const T *u = v_in + (long long)o + nb_off[a];
             T xr[VEC], xi[VEC];
-            ldv<T, VEC>(u, xr);
-            ldv<T, VEC>(u + blk, xi);
+            ldrow<T, VEC>(u, xr);
+            ldrow<T, VEC>(u + blk, xi);
             const T wg = nb_wg[a];
             v_axpy<VEC>(gr, wg, xr);
             v_axpy<VEC>(gi, wg, xi);
@@ -1204,8 +1252,8 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
             for (int a = n_d0; a < n_nb; ++a) {
                 const T *u = v_in + (long long)o + nb_off[a];
                 T xr[VEC], xi[VEC];
-                ldv<T, VEC>(u, xr);
-                ldv<T, VEC>(u + blk, xi);
+                ldrow<T, VEC>(u, xr);
+                ldrow<T, VEC>(u + blk, xi);
                 const T wg = nb_wg[a], wa = nb_wa[a];
                 v_axpy<VEC>(gr, wg, xr);
                 v_axpy<VEC>(gi, wg, xi);
@@ -1244,8 +1292,8 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
                         ii = ii < 0 ? ii + nq : ii - nq;
                     }
                     T xr[VEC], xi[VEC];
-                    ldv<T, VEC>(Ere + (size_t)ii * NP + l0, xr);
-                    ldv<T, VEC>(Ere + blk + (size_t)ii * NP + l0, xi);
+                    ldrow<T, VEC>(Ere + (size_t)ii * NP + l0, xr);
+                    ldrow<T, VEC>(Ere + blk + (size_t)ii * NP + l0, xi);
                     v_axpy<VEC>(gr, w * cq[b], xr);
                     v_axpy<VEC>(gi, w * cq[b], xi);
                 }
@@ -1307,8 +1355,8 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
         }
         if (want_pot && Pg) {  // potential term computed by another kernel
             T pr_[VEC], pi_[VEC];
-            ldv<T, VEC>(Pg + poff + (size_t)i * NP + l0, pr_);
-            ldv<T, VEC>(Pg + poff + blk + (size_t)i * NP + l0, pi_);
+            ldrow<T, VEC>(Pg + poff + (size_t)i * NP + l0, pr_);
+            ldrow<T, VEC>(Pg + poff + blk + (size_t)i * NP + l0, pi_);
 #pragma unroll
             for (int v = 0; v < VEC; ++v) {
                 ar[v] += pr_[v];
@@ -1326,8 +1374,8 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
         // ---- update -------------------------------------------------------------------------------
         if (!act) {
         } else if (mode == 0) {
-            stv<T, VEC>(v_out + o, ar);
-            stv<T, VEC>(v_out + o + blk, ai);
+            strow<T, VEC>(v_out + o, ar);
+            strow<T, VEC>(v_out + o + blk, ai);
         } else if (MIXED && e == 0) {
             const size_t o0 = (size_t)rep * g.tier0_rep_stride + (size_t)pr * 2 * blk + (size_t)i * NP + l0;
 #pragma unroll
@@ -1344,12 +1392,12 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
         } else {
             const T hh = sc.h;
             T br[VEC], bi[VEC];
-            ldv<T, VEC>(y + o, br);
-            ldv<T, VEC>(y + o + blk, bi);
+            ldrow<T, VEC>(y + o, br);
+            ldrow<T, VEC>(y + o + blk, bi);
             v_axpy<VEC>(br, hh, ar);
             v_axpy<VEC>(bi, hh, ai);
-            stv<T, VEC>(v_out + o, br);
-            stv<T, VEC>(v_out + o + blk, bi);
+            strow<T, VEC>(v_out + o, br);
+            strow<T, VEC>(v_out + o + blk, bi);
         }
     }
 }

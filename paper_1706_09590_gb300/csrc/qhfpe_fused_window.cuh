@@ -223,8 +223,8 @@ fused_window_kernel(GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<
         const size_t o0 = (size_t)rep * g.tier0_rep_stride + (size_t)pr * 2 * blk + (size_t)i * NP + l0;
         if (mode != 0) {
             if (tier0) {
-                ldv<double, VEC>(y0 + o0, b0r);
-                ldv<double, VEC>(y0 + o0 + blk, b0i);
+                ldrow<double, VEC>(y0 + o0, b0r);
+                ldrow<double, VEC>(y0 + o0 + blk, b0i);
             } else {
                 ldv<T, VEC>(y + o, br);
                 ldv<T, VEC>(y + o + blk, bi);
@@ -348,8 +348,8 @@ fused_window_kernel(GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<
             stv<T, VEC>(v_out + o, outr);
             stv<T, VEC>(v_out + o + blk, outi);
             if (mode == 2) {
-                stv<double, VEC>(y0_out + o0, b0r);
-                stv<double, VEC>(y0_out + o0 + blk, b0i);
+                strow<double, VEC>(y0_out + o0, b0r);
+                strow<double, VEC>(y0_out + o0 + blk, b0i);
             }
         } else {
             v_axpy<VEC>(br, sc.h, ar);
