@@ -344,8 +344,8 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
                         // the step's base: y itself at the first stage, the FP64 zeroth tier at the last
                         float br[VL], bi[VL];
                         if (k != 4 && (e != 0 || k != 1)) {
-                            ldv<float, VL>(yrow + go, br);
-                            ldv<float, VL>(yrow + go + blk, bi);
+                            ldrow<float, VL>(yrow + go, br);
+                            ldrow<float, VL>(yrow + go + blk, bi);
                         } else {
                             lds(pe, br);
                             lds(pe + PL4, bi);
@@ -453,14 +453,14 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
                             v_axpy<VL>(br, h, ar);
                             v_axpy<VL>(bi, h, ai);
                             if (k == 1) {
-                                stv<float, VL>(yrow + go, br);
-                                stv<float, VL>(yrow + go + blk, bi);
+                                strow<float, VL>(yrow + go, br);
+                                strow<float, VL>(yrow + go + blk, bi);
                             }
                         } else if (k != 1) {
                             // the FP64 zeroth tier as the sum of two floats (the rounded value and the rest)
                             float cr[VL], ci[VL];
-                            ldv<float, VL>(lrow, cr);
-                            ldv<float, VL>(lrow + blk, ci);
+                            ldrow<float, VL>(lrow, cr);
+                            ldrow<float, VL>(lrow + blk, ci);
                             v_axpy<VL>(cr, h, ar);
                             v_axpy<VL>(ci, h, ai);
                             v_add<VL>(br, cr);
@@ -479,8 +479,8 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
                                     split_double(w.y, bb[v + 1], low[v + 1]);
                                     if (traced) tr += w.x + w.y;
                                 }
-                                stv<float, VL>(lrow + off, low);
-                                stv<float, VL>(yrow + off, bb);
+                                strow<float, VL>(lrow + off, low);
+                                strow<float, VL>(yrow + off, bb);
                                 if (traced) sum += mud * tr;
                             };
                             accumulate(ar, br, 0, trr);
