@@ -909,6 +909,164 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
     }
 }
 
+// Phase B of one p-row of a warp where a lane has eight values (FP32 np 256): linear coupling, every term, lanes of
+// one p sign, the potential and the p-diagonal bath terms in xp (this lane's place of the row in X).  Bound by load
+// latency at 16 warps an SM.  The general loop below keeps the centre row and the p part of the tier coupling in
+// registers and has room for one neighbour in flight; here the p part goes straight to the sum, the centre row is
+// read again where the terminator needs it, and the neighbours come three at a time.  256 x 256, depth 10, three
+// states: 7.78 -> 7.03 ms a step (one neighbour at a time: 7.71; the base row loaded ahead of the p-stencil spills:
+// 7.65).
+template <int NP, bool MIXED>
+__device__ __forceinline__ void row_wide(const GridInfo &g, const StageScalars<float> &sc, const float *__restrict__ v_in,
+                                         const float *y, const double *y0, float *v_out, double *y0_out, double h, int mode,
+                                         bool tier0, size_t o, size_t o0, int i, const float *pcol, bool interior,
+                                         const long long *nb_off, const float *nb_wg, const float *nb_wa, int n_up,
+                                         int n_d0, int n_nb, bool term, const float2 *xp)
+{
+    constexpr int VEC = NP / 32, NB = 3;
+    const size_t blk = g.blk;
+    const int nq = g.nq;
+    const bool neg = pcol[0] < 0.f;
+    float ar[VEC], ai[VEC];
+    {  // -p dW/dq, 5th-order upwind
+        const float cneg[6] = {3, -30, -20, 60, -15, 2};  // p < 0: offsets -2..+3
+        const float cpos[6] = {-2, 15, -60, 20, 30, -3};  // p >= 0: offsets -3..+2
+        const int first = i - 3 + (neg ? 1 : 0);
+        const float *row = v_in + o - (size_t)i * NP;  // row 0
+        float kr[VEC], ki[VEC];
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) kr[v] = ki[v] = 0.f;
+#pragma unroll
+        for (int t0 = 0; t0 < 6; t0 += 3) {
+            float sr[3][VEC], si[3][VEC];
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                int ii = first + t0 + b;
+                bool ok = interior || (ii >= 0 && ii < nq);
+                if (!ok && g.periodic_q) {
+                    ii = ii < 0 ? ii + nq : ii - nq;
+                    ok = true;
+                }
+                if (ok) {
+                    ldrow<float, VEC>(row + (size_t)ii * NP, sr[b]);
+                    ldrow<float, VEC>(row + (size_t)ii * NP + blk, si[b]);
+                } else {
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) sr[b][v] = si[b][v] = 0.f;
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const float c = neg ? cneg[t0 + b] : cpos[t0 + b];
+                v_axpy<VEC>(kr, c, sr[b]);
+                v_axpy<VEC>(ki, c, si[b]);
+            }
+        }
+        float pk[VEC];
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) pk[v] = -(pcol[v] * sc.fkin);
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) {
+            ar[v] = pk[v] * kr[v];
+            ai[v] = pk[v] * ki[v];
+        }
+    }
+    {
+        float gr[VEC], gi[VEC];
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) gr[v] = gi[v] = 0.f;
+        const auto add = [&](int a, const float *xr, const float *xi) {
+            const float wg = nb_wg[a];
+            v_axpy<VEC>(gr, wg, xr);
+            v_axpy<VEC>(gi, wg, xi);
+            if (a >= n_d0) {
+                const float wa = nb_wa[a];
+                float q[VEC];
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) q[v] = wa * pcol[v];
+                v_fma<VEC>(ar, q, xr);
+                v_fma<VEC>(ai, q, xi);
+            }
+        };
+        int a = 0;
+#pragma unroll 1
+        for (; a + NB <= n_nb; a += NB) {
+            float xr[NB][VEC], xi[NB][VEC];
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                const float *u = v_in + (long long)o + nb_off[a + b];
+                ldrow<float, VEC>(u, xr[b]);
+                ldrow<float, VEC>(u + blk, xi[b]);
+            }
+#pragma unroll
+            for (int b = 0; b < NB; ++b) add(a + b, xr[b], xi[b]);
+        }
+#pragma unroll 1
+        for (; a < n_nb; ++a) {
+            float xr[VEC], xi[VEC];
+            const float *u = v_in + (long long)o + nb_off[a];
+            ldrow<float, VEC>(u, xr);
+            ldrow<float, VEC>(u + blk, xi);
+            add(a, xr, xi);
+        }
+        if (term) {  // d/dp (r_0 p W) of the terminator
+            float wr[VEC], wi[VEC], r0p[VEC];
+            ldrow<float, VEC>(v_in + o, wr);
+            ldrow<float, VEC>(v_in + o + blk, wi);
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) r0p[v] = sc.r0 * pcol[v];
+            v_fma<VEC>(gr, r0p, wr);
+            v_fma<VEC>(gi, r0p, wi);
+        }
+        if (n_nb > 0 || term) {  // 4th-order central d/dp, neighbours along p through the warp
+            const int left = (threadIdx.x + 31) & 31, right = (threadIdx.x + 1) & 31;
+            const auto ddp = [&](const float *x, float *acc) {
+                float er[VEC + 4];
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) er[v + 2] = x[v];
+                er[0] = __shfl_sync(0xffffffffu, x[VEC - 2], left);
+                er[1] = __shfl_sync(0xffffffffu, x[VEC - 1], left);
+                er[VEC + 2] = __shfl_sync(0xffffffffu, x[0], right);
+                er[VEC + 3] = __shfl_sync(0xffffffffu, x[1], right);
+#pragma unroll
+                for (int v = 0; v < VEC; ++v)
+                    acc[v] += sc.inv12dp * (er[v] - 8.f * er[v + 1] + 8.f * er[v + 3] - er[v + 4]);
+            };
+            ddp(gr, ar);
+            ddp(gi, ai);
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) {
+        ar[v] += xp[v].x;
+        ai[v] += xp[v].y;
+    }
+    if (mode == 0) {
+        strow<float, VEC>(v_out + o, ar);
+        strow<float, VEC>(v_out + o + blk, ai);
+    } else if (tier0) {
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) {
+            const double nr = y0[o0 + v] + h * (double)ar[v];
+            const double ni = y0[o0 + v + blk] + h * (double)ai[v];
+            v_out[o + v] = (float)nr;
+            v_out[o + v + blk] = (float)ni;
+            if (mode == 2) {
+                y0_out[o0 + v] = nr;
+                y0_out[o0 + v + blk] = ni;
+            }
+        }
+    } else {
+        float br[VEC], bi[VEC];
+        ldrow<float, VEC>(y + o, br);
+        ldrow<float, VEC>(y + o + blk, bi);
+        v_axpy<VEC>(br, sc.h, ar);
+        v_axpy<VEC>(bi, sc.h, ai);
+        strow<float, VEC>(v_out + o, br);
+        strow<float, VEC>(v_out + o + blk, bi);
+    }
+}
+
 // MULTI: one Horner stage of several propagators at once (heterogeneous batch: members differ in q
 // grid, surfaces, bath, hierarchy depth, closure, dt and replica count, and share NP, S and the
 // precision).  Blocks are numbered member by member; a block finds its member (first block numbers
@@ -1132,6 +1290,15 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
         const size_t poff = ebase + (size_t)pr * 2 * blk;
         const T *Vre = v_in + poff, *Vim = Vre + blk;
         const size_t o = poff + (size_t)i * NP + l0;
+        if constexpr (sizeof(T) == 4 && VEC >= 8 && !NL) {
+            if (uni_warp && fold && terms == QHFPE_TERM_ALL) {
+                row_wide<NP, MIXED>(g, sc, v_in, y, y0, v_out, y0_out, h, mode, MIXED && e == 0, o,
+                                    (size_t)rep * g.tier0_rep_stride + (size_t)pr * 2 * blk + (size_t)i * NP + l0, i, pcol,
+                                    interior, nb_off, nb_wg, nb_wa, n_up, n_d0, n_nb, term,
+                                    X + pad16((r * S2 + pr) * NP + l0));
+                continue;
+            }
+        }
         T ar[VEC], ai[VEC], wr[VEC], wi[VEC];
 #pragma unroll
         for (int v = 0; v < VEC; ++v) ar[v] = ai[v] = (T)0;
