@@ -297,11 +297,13 @@ qhfpe_status qhfpe_kernel_timing(qhfpe_t *h, int enable);
  * QHFPE_ETIMEOUT while the handle and the CUDA context stay usable. */
 qhfpe_status qhfpe_wait_selftest(qhfpe_t *h, int release, int limit_ms);
 /* Tile of the fused right-hand-side kernel (q rows per block) picked by the autotuner for the
- * handle's replicas: timed with CUDA events on the first propagation (0 before it, or when the
- * shape has no fused kernel; candidates 1, 2, 3, 4, 5, 6, 8, 12, 16 rows up to the kernel's
- * shared-memory limit, a power of two, and the q-window form's fixed tile, see qhfpe_stage_form).
+ * handle's replicas: timed with CUDA events on the first propagation (0 before it, when the shape has
+ * no fused kernel, or while the propagations run cluster-resident: small mixed-form two-state models with
+ * np 32 or 64; candidates 1, 2, 3, 4, 5, 6, 8, 12, 16 rows up to the kernel's shared-memory limit, levelled to
+ * equal tiles, and the q-window form's fixed tile, see qhfpe_stage_form).
  * The environment variable QHFPE_TILE_ROWS, when it holds a height from 1 to that limit, replaces
- * the timing with that tile (the q-window form then serves the shapes it applies to). */
+ * the timing with that tile (the q-window form then serves the shapes it applies to; no propagation runs
+ * cluster-resident, nor with QHFPE_RESIDENT=0). */
 qhfpe_status qhfpe_tile_rows(const qhfpe_t *h, int *rows);
 /* Persistent propagation (on = 1), Sec. III protocol on the device: every later run of RK4 steps of
  * the handle -- qhfpe_step and the propagations of qhfpe_response, whose phases pack all delays as
@@ -309,7 +311,7 @@ qhfpe_status qhfpe_tile_rows(const qhfpe_t *h, int *rows);
  * loop over the blocks of the fused stage kernel, grid-wide barriers separate the stages, and the
  * FP64 trace Tr{mu W^(0)} is reduced in the same launch after each step (fixed order).  Results equal
  * those of the graph-replayed launches (on = 0, the default) to rounding of the trace sums (the state is
- * the same arithmetic).  It covers the shapes with a fused kernel (np in {32, 64, 128, 256}, n_states
+ * the same arithmetic; against a cluster-resident run, equal to FP32 rounding of the stages).  It covers the shapes with a fused kernel (np in {32, 64, 128, 256}, n_states
  * <= 3), the FP64 and QHFPE_MIXED forms, the Condon dipole and the TRUNCATE / TERMINATOR closures; other
  * handles keep the graph replay.  Every barrier wait is bounded (2 s): when one gives up the call
  * returns QHFPE_ETIMEOUT and the handle turns sticky.  Kernel timing (qhfpe_kernel_timing) uses the

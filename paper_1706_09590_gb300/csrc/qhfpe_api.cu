@@ -1033,7 +1033,7 @@ qhfpe_status run_persistent(qhfpe *h, Prop &P, long n_steps, double *trace_dev, 
 
 // ---- resident propagation ------------------------------------------------------------------------
 // Mixed-form two-state propagators with np 32 or 64, linear coupling, no learned closure and the Condon
-// trace, whose lanes' eight p values share a sign.  QHFPE_RESIDENT=0 keeps the launch-per-stage form, as does
+// trace, whose lanes' p values share a sign.  QHFPE_RESIDENT=0 keeps the launch-per-stage form, as does
 // QHFPE_TILE_ROWS (which pins that form's tile) and kernel timing (which counts its launches).
 bool resident_wanted(const qhfpe *h, const Prop &P)
 {

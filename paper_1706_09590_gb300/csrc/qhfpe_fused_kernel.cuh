@@ -9,7 +9,8 @@
 //            digit-reversed order), multiplied by -i, and transformed back (sign -, natural order).
 //   phase B  one warp per p-row: upwind q-stencil (rows i-3..i+3 through L1/L2), damping and
 //            delta-term, tier-up/-down couplings (neighbour elements' rows), terminator, the
-//            potential term from shared memory, and out = base + h * L.
+//            potential term from shared memory, and out = base + h * L (row_wide: FP32 rows that fill a warp).
+// The FP64 form runs phase A and most of phase B on 64-bit integers (potential_fixed, rows_fixed).
 //
 // Grid order: the hierarchy element varies fastest, then the replica, then the q-tile, so the blocks
 // in flight cover all elements of a few q-tiles and the neighbour tiers and q-halos they re-read are
@@ -358,7 +359,8 @@ __device__ __forceinline__ void strow(T *p, const T *i)
 // 128-thread blocks (measured faster than 256: more independent blocks per SM keep phase A and phase B
 // of different blocks overlapping, and each barrier stalls four warps).  The kernel waits mostly on L2
 // loads, so resident warps count: FP32 with one or two states runs seven blocks per SM (72 registers;
-// measured 5 % faster than six at 80), three states six (seven would spill), NP = 256 four (wider rows).
+// measured 5 % faster than six at 80), three states six (seven would spill), NP = 256 four (wider rows; 256 x 256 with
+// three states took 34.4 ms for four steps with four, 35.7 with three, 43.2 with five, which spill).
 // FP64 (integer arithmetic, latency-bound below 16 warps) runs four at 128 registers: on 96 x 128 at depth 8
 // three, four and five blocks took within 3 % of each other, two 25 % longer.
 template <typename T, int NP, int S>
@@ -704,7 +706,7 @@ __device__ __forceinline__ FixedWeight fixed_weight(double w)
 
 // Phase B of the FP64 form (linear coupling, all terms, the potential and the p-diagonal bath terms already
 // in X): kinetic term, tier couplings and update of the block's rows.  As in the transforms
-// (qhfpe_fixed.cuh) the FP64 pipe would bound it, so the sums run on 64-bit integers:
+// (qhfpe_fixed.cuh) the FP64 pipe would bound it, so it is left with the tier sums:
 //   kinetic  the q differences have small integer weights (sum of sizes 130).  A warp takes four rows of one
 //            pair; for each of its p columns the nine rows read are brought to the column's largest exponent
 //            (62 bits below it) once, and the four sums of six are exact.  Where the rows' own exponents are
@@ -909,13 +911,13 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
     }
 }
 
-// Phase B of one p-row of a warp where a lane has eight values (FP32 np 256): linear coupling, every term, lanes of
-// one p sign, the potential and the p-diagonal bath terms in xp (this lane's place of the row in X).  Bound by load
-// latency at 16 warps an SM.  The general loop below keeps the centre row and the p part of the tier coupling in
-// registers and has room for one neighbour in flight; here the p part goes straight to the sum, the centre row is
-// read again where the terminator needs it, and the neighbours come three at a time.  256 x 256, depth 10, three
-// states: 7.78 -> 7.03 ms a step (one neighbour at a time: 7.71; the base row loaded ahead of the p-stencil spills:
-// 7.65).
+// Phase B of one p-row that fills a warp (FP32, np 128 and 256): linear coupling, every term, lanes of one p sign, the
+// potential and the p-diagonal bath terms in xp (this lane's place of the row in X).  Bound by load latency at 16 to
+// 28 warps an SM.  The general loop below keeps the centre row and the p part of the tier coupling in registers
+// and has one neighbour in flight; here the p part goes straight to the sum, the centre row is read again where the
+// terminator needs it, and the neighbours come three at a time.  256 x 256, depth 10, three states: 7.78 -> 7.03 ms
+// a step (one neighbour at a time: 7.71; the base row loaded ahead of the p-stencil spills: 7.65).  np 128: 512 x
+// 128, two states 86 -> 83 us, 96 x 128, three states, depth 4 196 -> 187 us.
 template <int NP, bool MIXED>
 __device__ __forceinline__ void row_wide(const GridInfo &g, const StageScalars<float> &sc, const float *__restrict__ v_in,
                                          const float *y, const double *y0, float *v_out, double *y0_out, double h, int mode,
@@ -1290,7 +1292,7 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
         const size_t poff = ebase + (size_t)pr * 2 * blk;
         const T *Vre = v_in + poff, *Vim = Vre + blk;
         const size_t o = poff + (size_t)i * NP + l0;
-        if constexpr (sizeof(T) == 4 && VEC >= 8 && !NL) {
+        if constexpr (sizeof(T) == 4 && NP >= 128 && !NL) {
             if (uni_warp && fold && terms == QHFPE_TERM_ALL) {
                 row_wide<NP, MIXED>(g, sc, v_in, y, y0, v_out, y0_out, h, mode, MIXED && e == 0, o,
                                     (size_t)rep * g.tier0_rep_stride + (size_t)pr * 2 * blk + (size_t)i * NP + l0, i, pcol,

@@ -10,9 +10,9 @@
 // live in shared memory; the step's base y (8 B per cell and stage, coalesced) and the FP64 zeroth tier
 // stay in global memory, L2-resident.
 //
-// Inside a block there is no barrier at all: a row of one pair belongs to np/8 lanes, eight consecutive p
-// values each, the four pairs of a row to neighbouring lane groups of one warp.
-//   FFT along p  length-np/8 transform across the lanes (radix 2, shuffles), twiddles, length 8 in registers;
+// Inside a block there is no barrier at all: a row of one pair belongs to eight lanes with np/8 consecutive p
+// values each (res_lane), the four pairs of a row to neighbouring lane groups of one warp.
+//   FFT along p  length-8 transform across the lanes (radix 2, shuffles), twiddles, length np/8 in registers;
 //                the inverse runs back the same way, so every lane ends with its own p values
 //   mixing       the r-space products with the other pairs' values by shuffles; tables per lane, shared by the
 //                elements of a row
