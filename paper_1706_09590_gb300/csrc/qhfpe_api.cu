@@ -603,8 +603,10 @@ qhfpe_status build_model(qhfpe *h, Model &M, int S, const double *U, const doubl
             int k = -4096;  // a row of zeros: below every other term
             if (big > 0.0) std::frexp(big, &k);
             kx[r] = k;
+            const bool plain = std::abs(k) < 900;  // 2^(62 - k) is a normal double: the product is exact
+            const double scale = plain ? std::ldexp(1.0, 62 - k) : 0.0;
             for (int t = 0; t < p.np; ++t) {
-                const long long c = big > 0.0 ? std::llrint(std::ldexp(row[t], 62 - k)) : 0;
+                const long long c = big > 0.0 ? std::llrint(plain ? row[t] * scale : std::ldexp(row[t], 62 - k)) : 0;
                 std::memcpy(row + t, &c, sizeof(c));
             }
         }
