@@ -610,10 +610,10 @@ qhfpe_status build_model(qhfpe *h, Model &M, int S, const double *U, const doubl
                 std::memcpy(row + t, &c, sizeof(c));
             }
         }
-        ft.resize(3 * M.tab_n + 3 * p.np + kx.size() / 2);
-        std::memcpy(ft.data() + 3 * M.tab_n + 3 * p.np, kx.data(), kx.size() * sizeof(int));
-        QH_CK(h, dalloc(&M.ftab64, ft.size()));
-        QH_CK(h, cudaMemcpyAsync(M.ftab64, ft.data(), sizeof(double) * ft.size(), cudaMemcpyHostToDevice, st));
+        const size_t ft_n = 3 * M.tab_n + 3 * p.np;
+        QH_CK(h, dalloc(&M.ftab64, ft_n + kx.size() / 2));
+        QH_CK(h, cudaMemcpyAsync(M.ftab64, ft.data(), sizeof(double) * ft_n, cudaMemcpyHostToDevice, st));
+        QH_CK(h, cudaMemcpyAsync(M.ftab64 + ft_n, kx.data(), sizeof(int) * kx.size(), cudaMemcpyHostToDevice, st));
         QH_CK(h, dalloc(&M.ftab32, ft32.size()));
         QH_CK(h, cudaMemcpyAsync(M.ftab32, ft32.data(), sizeof(float) * ft32.size(), cudaMemcpyHostToDevice, st));
         QH_CK(h, (prepare_fused<float, true>(p.np, S)));
@@ -889,8 +889,9 @@ qhfpe_status autotune(qhfpe *h, Prop &P)
     QH_CK(h, cudaEventCreate(&a));
     QH_CK(h, cudaEventCreate(&b));
     float best = 1e30f, ms = 0.f;
-    // right-hand sides of every replica into vB with the given form and tile: one to warm up, one timed, and two
-    // more unless that one was far behind the best so far; *ms for three
+    // stages of every replica into vB with the given form and tile, with a base read as in a step (vA, whatever it
+    // holds, times one plus nothing: without it the general form looked 4 % faster than it is in steps of 96 x 128
+    // models): one to warm up, one timed, and two more unless that one was far behind the best so far; *ms for three
     auto time_one = [&](int form, int tq, float *ms) -> qhfpe_status {
         *ms = 0.f;
         for (int n : {1, 2}) {
@@ -898,12 +899,12 @@ qhfpe_status autotune(qhfpe *h, Prop &P)
                 if (rep == 0) QH_CK(h, cudaEventRecord(a, st));
                 cudaError_t e;
                 if (P.mixed)
-                    e = launch_fused<float, true>(P.g, M.elems, M.f32(), (const float *)P.y, (const float *)P.y, P.y0,
-                                                  (float *)P.vB, nullptr, 0.0, 0, QHFPE_TERM_ALL, 0, P.g.n_rep, st,
+                    e = launch_fused<float, true>(P.g, M.elems, M.f32(), (const float *)P.y, (const float *)P.vA, P.y0,
+                                                  (float *)P.vB, nullptr, 0.0, 1, QHFPE_TERM_ALL, 0, P.g.n_rep, st,
                                                   P.tc ? (const float *)P.P : nullptr, tq, form);
                 else
-                    e = launch_fused<double, false>(P.g, M.elems, M.f64(), (const double *)P.y, (const double *)P.y,
-                                                    nullptr, (double *)P.vB, nullptr, 0.0, 0, QHFPE_TERM_ALL, 0, P.g.n_rep,
+                    e = launch_fused<double, false>(P.g, M.elems, M.f64(), (const double *)P.y, (const double *)P.vA,
+                                                    nullptr, (double *)P.vB, nullptr, 0.0, 1, QHFPE_TERM_ALL, 0, P.g.n_rep,
                                                     st, nullptr, tq, form);
                 QH_CK(h, e);
             }
