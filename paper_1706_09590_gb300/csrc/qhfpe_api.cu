@@ -374,6 +374,14 @@ cudaError_t dalloc(T **p, size_t n)
     return cudaMalloc((void **)p, n * sizeof(T) + 16);
 }
 
+// Upload of pageable host data that kernels on any stream may read on return.  (A plain cudaMemcpy runs on the
+// default stream and may return with the data only staged; the handles' streams don't wait for that stream.)
+cudaError_t upload(void *dst, const void *src, size_t bytes, cudaStream_t st)
+{
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    return e ? e : cudaStreamSynchronize(st);
+}
+
 // Potential tables (Eq. (quantum-liouvillian) in r-space) for an FFT's output order, pre-scaled by
 // 1/np.  freq(pos) gives the frequency index sitting at position pos; n_tw twiddles e^{2 pi i t/np}.
 template <typename F>
@@ -992,7 +1000,7 @@ qhfpe_status persistent_desc(qhfpe *h, Prop &P)
     x.y0 = P.mixed ? P.y0 : nullptr;
     x.block0 = 0;
     QH_CK(h, cudaMalloc(&P.pdesc, sizeof(x)));
-    QH_CK(h, cudaMemcpy(P.pdesc, &x, sizeof(x), cudaMemcpyHostToDevice));
+    QH_CK(h, upload(P.pdesc, &x, sizeof(x), h->stream));
     QH_CK(h, cudaMalloc((void **)&P.pbar, 4 * sizeof(unsigned)));
     P.pdesc_tq = tq;
     return QHFPE_OK;
@@ -1090,15 +1098,20 @@ bool resident_plan(const std::vector<const Prop *> &props, ResidentPlan &R)
     return found;
 }
 
-qhfpe_status resident_tables(qhfpe *h, Model &M, const double *U)
+// (complete on return: the model's next run may be on another stream, a batch's on its first member's)
+qhfpe_status resident_tables(qhfpe *h, Model &M, const double *U, cudaStream_t st)
 {
     if (M.rtab) return QHFPE_OK;
     std::vector<double> t;
     const int np = M.np;
     build_tables(M, U, t, [np](int pos) { return resident_frequency(np, pos); }, 0, true);
     std::vector<float> f(t.begin(), t.end());
-    QH_CK(h, dalloc(&M.rtab, f.size()));
-    QH_CK(h, cudaMemcpy(M.rtab, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice));
+    float *d = nullptr;
+    QH_CK(h, dalloc(&d, f.size()));
+    const cudaError_t e = upload(d, f.data(), f.size() * sizeof(float), st);
+    if (e) cudaFree(d);
+    QH_CK(h, e);
+    M.rtab = d;
     return QHFPE_OK;
 }
 
@@ -1185,7 +1198,7 @@ qhfpe_status run_steps(qhfpe *h, Prop &P, long n_steps, double *trace_dev, long 
         else QH_CK(h, launch_trace<double>(P.g, (const double *)P.y, P.g.rep_stride, P.m->mu, P.sink, 1, P.partial, st, P.m->trace_mu_q()));
     }
     if (resident) {
-        qhfpe_status r = resident_tables(h, *P.m, h->U.data());
+        qhfpe_status r = resident_tables(h, *P.m, h->U.data(), st);
         if (r != QHFPE_OK) return r;
         return run_resident(h, {&P}, record ? std::vector<double *>{trace_dev} : std::vector<double *>{}, stride, P.res,
                             n_steps, st);
@@ -2478,7 +2491,7 @@ qhfpe_status batch_upload(qhfpe_batch *b, int tq)
     }
     if (blocks > 0x7fffffffL) return h0->fail(QHFPE_EUNSUPPORTED, "batch: more than 2^31 - 1 blocks per stage");
     if (!b->desc) QH_CK(h0, cudaMalloc(&b->desc, d.size() * sizeof(MultiMember<T>)));
-    QH_CK(h0, cudaMemcpy(b->desc, d.data(), d.size() * sizeof(MultiMember<T>), cudaMemcpyHostToDevice));
+    QH_CK(h0, ::upload(b->desc, d.data(), d.size() * sizeof(MultiMember<T>), h0->stream));
     b->blocks = blocks;
     return QHFPE_OK;
 }
@@ -2649,7 +2662,7 @@ qhfpe_status qhfpe_batch_step(qhfpe_batch_t *b, long n_steps, double *const *tra
         std::vector<Prop *> props;
         std::vector<double *> traces;
         for (qhfpe *h : b->mem) {
-            if ((r = resident_tables(h, *h->model, h->U.data())) != QHFPE_OK) return r;
+            if ((r = resident_tables(h, *h->model, h->U.data(), st)) != QHFPE_OK) return r;
             props.push_back(h->main.get());
             if (record) traces.push_back(h->main->trace_buf);
         }
