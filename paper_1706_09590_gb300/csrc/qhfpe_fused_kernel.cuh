@@ -762,8 +762,8 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                     int ii = ia + first + t;
                     bool ok = t < nr + 5 && ii >= 0 && ii < nq;
                     if (!ok && g.periodic_q && t < nr + 5) {
-                        ii = ii < 0 ? ii + nq : ii - nq;
-                        ok = ii >= 0 && ii < nq;
+                        ii = wrap_q(ii, nq);
+                        ok = true;
                     }
                     return ok ? V[(size_t)ii * NP + l0 + v] : 0.0;
                 };
@@ -946,7 +946,7 @@ __device__ __forceinline__ void row_wide(const GridInfo &g, const StageScalars<f
                 int ii = first + t0 + b;
                 bool ok = interior || (ii >= 0 && ii < nq);
                 if (!ok && g.periodic_q) {
-                    ii = ii < 0 ? ii + nq : ii - nq;
+                    ii = wrap_q(ii, nq);
                     ok = true;
                 }
                 if (ok) {
@@ -1330,7 +1330,7 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
                     int ii = i + t0 + b - 3 + sh;
                     bool ok = ii >= 0 && ii < nq;
                     if (!ok && g.periodic_q) {
-                        ii = ii < 0 ? ii + nq : ii - nq;
+                        ii = wrap_q(ii, nq);
                         ok = true;
                     }
                     if (ok) {
@@ -1371,7 +1371,7 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
                     int ii = i + d;
                     if (ii < 0 || ii >= nq) {
                         if (!g.periodic_q) continue;
-                        ii = ii < 0 ? ii + nq : ii - nq;
+                        ii = wrap_q(ii, nq);
                     }
                     T rr[VEC], ri[VEC];
                     ldrow<T, VEC>(Vre + (size_t)ii * NP + l0, rr);
@@ -1458,7 +1458,7 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
                     int ii = i + dqo[b];
                     if (ii < 0 || ii >= nq) {
                         if (!g.periodic_q) continue;
-                        ii = ii < 0 ? ii + nq : ii - nq;
+                        ii = wrap_q(ii, nq);
                     }
                     T xr[VEC], xi[VEC];
                     ldrow<T, VEC>(Ere + (size_t)ii * NP + l0, xr);

@@ -157,8 +157,8 @@ fused_window_kernel(GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<
             int ii = ia - 3 + b0 + b;
             bool ok = ii >= 0 && ii < nq;
             if (!ok && g.periodic_q) {
-                ii = ii < 0 ? ii + nq : ii - nq;
-                ok = ii >= 0 && ii < nq;
+                ii = wrap_q(ii, nq);
+                ok = true;
             }
             if (ok) {
                 ldv<T, VEC>(Vre + (size_t)ii * NP + l0, wr_[b]);

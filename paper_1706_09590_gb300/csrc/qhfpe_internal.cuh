@@ -77,6 +77,17 @@ struct FusedTables {
     const int *kx;
 };
 
+#ifdef __CUDACC__
+// q row ii of the periodic axis, -3 <= ii < nq + 3 and beyond: nq may be smaller than the stencils' reach, so that
+// one period is not always enough
+__device__ __forceinline__ int wrap_q(int ii, int nq)
+{
+    while (ii < 0) ii += nq;
+    while (ii >= nq) ii -= nq;
+    return ii;
+}
+#endif
+
 // Scalars of one fused stage launch, rounded once on the host: 1/(12 dp), 1/(60 dq), the delta-term and
 // terminator coefficients of the 5-point d2/dp2, r_0 and the Horner step h.
 template <typename T>

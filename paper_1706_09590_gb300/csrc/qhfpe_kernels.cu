@@ -56,7 +56,7 @@ stage_kernel(GridInfo g, const ElemInfo *__restrict__ elems, const T *__restrict
         auto ld = [&](int ii, T c) {
             if (ii < 0 || ii >= nq) {
                 if (!g.periodic_q) return;
-                ii = ii < 0 ? ii + nq : ii - nq;
+                ii = wrap_q(ii, nq);
             }
             size_t o = (size_t)ii * np + l;
             sr += c * V[o];

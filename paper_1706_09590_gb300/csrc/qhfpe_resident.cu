@@ -221,7 +221,7 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
     for (int t = threadIdx.x; t < E * 4 * 2 * RH * (NP / 4); t += blockDim.x) {
         const int q = t % (NP / 4), r = (t / (NP / 4)) % RH, pp = t / (NP / 4) / RH;  // pp: (elem, pair, plane)
         int i = lo + r - 3;
-        if (g.periodic_q) i = i < 0 ? i + nq : (i >= nq ? i - nq : i);
+        if (g.periodic_q) i = wrap_q(i, nq);
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (i >= 0 && i < nq && r < nloc + 6)
             v = *reinterpret_cast<const float4 *>(yrep + (size_t)(pp / 2) * 2 * blk + (size_t)(pp & 1) * blk + (size_t)i * NP + 4 * q);
@@ -290,10 +290,12 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
         lrow = lrep + c;
         y0row = y0rep + c;
         n_halo = 0;
-        // the row on the unwrapped axis (periodic q: also a period away); block t holds t R - 3 .. t R + R + 2,
-        // so at most six others hold a row (three on each side at one row a block)
+        // the row on the unwrapped axis (periodic q: also whole periods away, as far as the three rows beyond either
+        // edge reach: one where nq >= 3); block t holds t R - 3 .. t R + R + 2, so at most six others hold a row
+        // (three on each side at one row a block)
         const int blocks = (nq + R - 1) / R;
-        for (int w = g.periodic_q ? -1 : 0; w <= (g.periodic_q ? 1 : 0); ++w) {
+        const int periods = g.periodic_q ? (nq + 2) / nq : 0;
+        for (int w = -periods; w <= periods; ++w) {
             const int pos = i + w * nq;
             for (int t = 0; t < blocks; ++t) {
                 const int at = pos - t * R + 3;
