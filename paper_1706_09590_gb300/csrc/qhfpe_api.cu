@@ -876,7 +876,8 @@ qhfpe_status step_dispatch(qhfpe *h, Prop &P, bool record)
 // Autotuner of the fused stage kernel's tile (q rows per block): each candidate evaluates the full
 // right-hand side of every replica (into a stage buffer, which holds no data between steps) a few
 // times, timed with CUDA events on the handle's stream; the fastest is kept for this propagator.
-// Results do not depend on the tile (every cell is computed by the same arithmetic).
+// Results do not depend on the tile (every cell is computed by the same arithmetic), only on the form: the q-window kernel
+// adds a cell's FP32 terms in another order than the general one.
 qhfpe_status autotune(qhfpe *h, Prop &P)
 {
     const Model &M = *P.m;
@@ -943,15 +944,19 @@ qhfpe_status autotune(qhfpe *h, Prop &P)
     bool timed[17] = {};
     for (int c : {first, 1, 2, 3, 4, 5, 6, 8, 12, 16}) {
         if (c > tmax) break;
-        const int tiles = (P.g.nq + c - 1) / c, tq = (P.g.nq + tiles - 1) / tiles;  // as many tiles, of one height
-        if (timed[tq]) continue;
-        timed[tq] = true;
-        qhfpe_status r = time_one(0, tq, &ms);
-        if (r != QHFPE_OK) return r;
-        if (ms < best) {
-            best = ms;
-            best_tq = tq;
-            best_form = 0;
+        const int tiles = (P.g.nq + c - 1) / c, level = (P.g.nq + tiles - 1) / tiles;  // as many tiles, of one height
+        for (int tq : {level, c}) {
+            // the FP64 form works on groups of four q rows of the grid: multiples of four as they are, too (97 rows of
+            // one state, np 128: tiles of 14 rows 23.1 ms for an equilibration, of 16 rows 22.5)
+            if (timed[tq] || (tq != level && (P.mixed || tq % 4 != 0))) continue;
+            timed[tq] = true;
+            qhfpe_status r = time_one(0, tq, &ms);
+            if (r != QHFPE_OK) return r;
+            if (ms < best) {
+                best = ms;
+                best_tq = tq;
+                best_form = 0;
+            }
         }
     }
     cudaEventDestroy(a);

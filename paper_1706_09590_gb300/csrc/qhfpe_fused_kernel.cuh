@@ -710,7 +710,10 @@ __device__ __forceinline__ FixedWeight fixed_weight(double w)
 //   kinetic  the q differences have small integer weights (sum of sizes 130).  A warp takes four rows of one
 //            pair; for each of its p columns the nine rows read are brought to the column's largest exponent
 //            (62 bits below it) once, and the four sums of six are exact.  Where the rows' own exponents are
-//            more than eight apart each of the four takes its own.
+//            more than eight apart each of the four takes its own.  The four are rows 4 n .. 4 n + 3 of the grid:
+//            a unit that holds only some of them, at the edge of a tile or in a small one, reads all nine rows
+//            all the same, so that results don't depend on the tile.  (With an exponent for each row everywhere
+//            four steps of 96 x 128 at depth 8 took 9.26 ms, this way 8.11.)
 //   tiers    G = sum of the neighbours' rows, weighted, in FP64 (one instruction per value and neighbour, on a
 //            pipe that has room for them; in integers the conversions alone took twenty); its row is brought
 //            to the largest exponent, 57 bits below it, and the p difference (weights 1, 8) is exact.
@@ -741,12 +744,15 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
     }
     const int first = neg ? -2 : -3;
     const double bad = bitsd(0x7ff8000000000000ull);
-    const int rg = min(RG, (rows * S2 + FTHREADS / 32 - 1) / (FTHREADS / 32));  // fewer where warps would idle
+    int rg = min(RG, (rows * S2 + FTHREADS / 32 - 1) / (FTHREADS / 32));  // fewer where warps would idle
+    rg = rg == 3 ? RG : rg;
+    const int u0 = i0 / rg, n_u = (i0 + rows - 1) / rg - u0 + 1;  // units of rg rows, aligned on the grid
 #pragma unroll 1
-    for (int u = warp; u < ((rows + rg - 1) / rg) * S2; u += FTHREADS / 32) {
-        const int pr = u % S2, r0 = (u / S2) * rg;
-        const int nr = min(rg, rows - r0);
-        const int ia = i0 + r0;
+    for (int u = warp; u < n_u * S2; u += FTHREADS / 32) {
+        const int pr = u % S2, us = (u0 + u / S2) * rg;
+        const int ia = max(us, i0), r0 = ia - i0;
+        const int nr = min(us + rg, i0 + rows) - ia;
+        const int gs = ia & ~(RG - 1), k0 = ia - gs;  // the group of RG grid rows that the unit's are among
         const size_t poff = ebase + (size_t)pr * 2 * blk;
 #pragma unroll 1
         for (int plane = 0; plane < 2; ++plane) {
@@ -759,9 +765,9 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
             for (int v = 0; v < VEC; ++v) {  // (one p column at a time: more in flight would only lengthen the code)
                 const FixedWeight pk = fixed_weight(-(pgrid[l0 + v] * sc.fkin));
                 const auto value = [&](int t) {  // window row t of the column
-                    int ii = ia + first + t;
-                    bool ok = t < nr + 5 && ii >= 0 && ii < nq;
-                    if (!ok && g.periodic_q && t < nr + 5) {
+                    int ii = gs + first + t;
+                    bool ok = ii >= 0 && ii < nq;
+                    if (!ok && g.periodic_q) {
                         ii = wrap_q(ii, nq);
                         ok = true;
                     }
@@ -799,26 +805,27 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
 #pragma unroll
                 for (int r = 0; r < RG; ++r) {
                     const int er = max(max(max(ex[r], ex[r + 1]), max(ex[r + 2], ex[r + 3])), max(ex[r + 4], ex[r + 5]));
-                    if (r < nr) least = min(least, er);
+                    if (gs + r < nq) least = min(least, er);
                 }
                 if (!__any_sync(0xffffffffu, E - least > 8)) {
                     Half x[RG + 5];
 #pragma unroll
-                    for (int t = 0; t < RG + 5; ++t) x[t] = halves(to_fixed<62>(raw[t], E));
+                    for (int t = 0; t < RG + 5; ++t)
+                        x[t] = halves(to_fixed<62>(raw[t], E));
 #pragma unroll
                     for (int r = 0; r < RG; ++r)
-                        if (r < nr) emit(r, x + r, E);
+                        if (r >= k0 && r < k0 + nr) emit(r - k0, x + r, E);
                 } else {  // steep in q: an exponent for each row
 #pragma unroll
                     for (int r = 0; r < RG; ++r) {
-                        if (r >= nr) continue;
+                        if (r < k0 || r >= k0 + nr) continue;
                         int er = EXP_MIN;
 #pragma unroll
                         for (int t = 0; t < 6; ++t) er = max(er, ex[r + t]);
                         Half x[6];
 #pragma unroll
                         for (int t = 0; t < 6; ++t) x[t] = halves(to_fixed<62>(raw[r + t], er));
-                        emit(r, x, er);
+                        emit(r - k0, x, er);
                     }
                 }
             }
