@@ -1156,9 +1156,8 @@ qhfpe_status run_resident(qhfpe *h, const std::vector<Prop *> &props, const std:
             x.tw = P.m->f32().tw;
             x.sc[0] = stage_scalars<float>(P.g, 0.0);
             for (int k = 1; k <= 4; ++k) x.sc[k] = stage_scalars<float>(P.g, P.dt / k);
-            x.dt = P.dt;
+            for (int k = 1; k <= 4; ++k) x.hd[k] = P.dt / k;
             x.y = (float *)P.y;
-            x.lo = (float *)P.vB;
             x.y0 = P.y0;
             x.mu = P.m->mu;
             x.part = record ? R.part + part : nullptr;
@@ -1169,7 +1168,7 @@ qhfpe_status run_resident(qhfpe *h, const std::vector<Prop *> &props, const std:
         }
         QH_CK(h, cudaMemcpyAsync(R.desc, d.data(), d.size() * sizeof(ResidentMember), cudaMemcpyHostToDevice, st));
         QH_CK(h, launch_resident(np, (const ResidentMember *)R.desc, (int)d.size(), R.clusters, R.csize, R.threads, R.smem,
-                                 len, done == 0, st));
+                                 len, st));
         if (record)
             for (size_t m = 0; m < props.size(); ++m)
                 QH_CK(h, launch_resident_trace(d[m].part, props[m]->g.n_rep, len, n_part, props[m]->g.dq * props[m]->g.dp,

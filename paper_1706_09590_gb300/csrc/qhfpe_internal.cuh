@@ -216,9 +216,9 @@ struct ResidentMember {
     const float *tab;         // D | L | R [S][S][nq][np] and lpp [np] in the resident transform's order
     const float *tw;          // np twiddles
     StageScalars<float> sc[5];  // [k]: stage k = 1..4 (h = dt / k)
-    double dt;
-    float *y, *lo;            // FP32 state; low halves of its FP64 zeroth tier, same layout
-    double *y0;
+    double hd[5];             // [k]: dt / k, for the FP64 zeroth tier
+    float *y;                 // FP32 state
+    double *y0;               // its FP64 zeroth tier
     const double *mu;
     double *part;             // trace parts [n_rep][n_steps][warps of a cluster] complex, or nullptr
     int cluster0;
@@ -230,9 +230,9 @@ size_t resident_smem(int np, int n_elem, int rows);  // 0: a block cannot have t
 int resident_threads(int np, int n_elem, int rows);
 // clusters of csize blocks that fit on the device at once (0: that size cannot run)
 cudaError_t resident_capacity(int np, int csize, int threads, size_t smem, int *clusters);
-// n_steps RK4 steps of every member (device array, cluster0 ascending from 0); first: (re)compute lo
+// n_steps RK4 steps of every member (device array, cluster0 ascending from 0)
 cudaError_t launch_resident(int np, const ResidentMember *members, int n_mem, int clusters, int csize, int threads,
-                            size_t smem, int n_steps, bool first, cudaStream_t st);
+                            size_t smem, int n_steps, cudaStream_t st);
 cudaError_t launch_resident_trace(const double *part, int n_rep, int n_steps, int n_part, double scale, double *out,
                                   long stride, long slot0, cudaStream_t st);
 

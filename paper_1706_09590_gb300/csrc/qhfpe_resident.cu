@@ -18,15 +18,15 @@
 //                elements of a row
 //   the rest     q rows by 16-byte shared-memory loads, the p difference with two values from each
 //                neighbouring lane
-// The arithmetic is the fused stage kernel's (FP32 stages, FP64 accumulation of the zeroth tier).
+// The arithmetic is the fused stage kernel's: FP32 stages, the zeroth tier's base and update in FP64 at every stage.
 #include "qhfpe.h"
 #include "qhfpe_fused_kernel.cuh"
 
 namespace {
 
 // consecutive p values of a lane, and threads of a block: four values at np = 32 (128 registers, 16 warps
-// per SM: 37 us a step for 76 replicas of four elements on 32 x 32, 12.4 us for one; eight values at 248
-// registers and 8 warps took 41.5 and 18.4 us)
+// per SM: 37 us a step for 76 replicas of four elements on 32 x 32, 13.5 us for one; eight values at 248
+// registers and 8 warps took 10 and 50 % longer)
 constexpr int res_lane(int np) { return np == 32 ? 4 : 8; }
 constexpr int res_threads(int np) { return np == 32 ? 512 : 256; }
 constexpr int RES_MAXNB = 2 * QH_MAX_MODES;
@@ -125,38 +125,25 @@ template <int LPR, int VL> __device__ __forceinline__ void lanes_inverse(float2 
     }
 }
 
-// An FP64 value as the nearest float and the rest, by integer operations (GB300 converts two a clock and SM):
-// floats below 2^-126 are taken as zero.
-__device__ __forceinline__ void split_double(double w, float &hi, float &lo)
+// Conversions by integer operations (GB300 converts two values a clock and SM); the instruction serves floats below
+// 2^-126, values beyond the floats, infinities and NaN.  double to float, to nearest even:
+__device__ __forceinline__ float narrow(double w)
 {
     const unsigned h = (unsigned)__double2hiint(w), l = (unsigned)__double2loint(w);
-    const int ex = (int)((h >> 20) & 2047u);
-    if (ex > 1150) {  // beyond the floats, infinite or NaN
-        hi = (float)w;
-        lo = 0.f;
-        return;
-    }
+    const unsigned ex = (h >> 20) & 2047u;
+    if (ex - 897u > 253u && (h << 1 | l) != 0u) return (float)w;
     const unsigned rest = l & 0x1fffffffu;
-    unsigned f = __funnelshift_l(l, (h & 0x7fffffffu) - 0x38000000u, 3);
+    const unsigned f = __funnelshift_l(l, (h & 0x7fffffffu) - 0x38000000u, 3);
     const unsigned up = (rest > 0x10000000u || (rest == 0x10000000u && (f & 1u))) ? 1u : 0u;
-    f += up;
-    const float unit = __uint_as_float((unsigned)max(ex - 948, 0) << 23);  // 2^(ex - 1075)
     const unsigned s = h & 0x80000000u;
-    const float r = (float)((int)rest - (int)(up << 29)) * unit;
-    hi = __uint_as_float(ex < 897 ? s : (f | s));
-    lo = ex < 897 ? 0.f : __uint_as_float(__float_as_uint(r) ^ s);
+    return __uint_as_float(ex == 0u ? s : ((f + up) | s));
 }
-// a float as a double, by integer operations (below 2^-126: zero)
 __device__ __forceinline__ double widen(float a)
 {
     const unsigned u = __float_as_uint(a), m = u & 0x7fffffffu;
-    unsigned h = (u & 0x80000000u) | ((m >> 3) + 0x38000000u), l = u << 29;
-    if (m >= 0x7f800000u) h |= 0x7ff00000u;
-    if (m < 0x00800000u) {
-        h = u & 0x80000000u;
-        l = 0;
-    }
-    return __hiloint2double((int)h, (int)l);
+    if (m - 0x00800000u > 0x7effffffu && m != 0u) return (double)a;
+    const unsigned h = (u & 0x80000000u) | (m == 0u ? 0u : (m >> 3) + 0x38000000u);
+    return __hiloint2double((int)h, (int)(u << 29));
 }
 
 template <int NP>
@@ -209,7 +196,6 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
         o.fpp = M.sc[0].fdelta + (I.terminator ? M.sc[0].fterm : 0.f);
     }
     float *yrep = M.y + (size_t)rep * g.rep_stride;
-    float *lrep = M.lo + (size_t)rep * g.rep_stride;
     double *y0rep = M.y0 + (size_t)rep * g.tier0_rep_stride;
     const size_t blk = g.blk;
 
@@ -268,7 +254,6 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
     const float *tP = M.tab + 3 * tabn + l0;                                                      // eigenvalues of d2/dp2
     const double mud = M.mu[(pair & 1) * 2 + (pair >> 1)];                                        // Tr{mu W}: mu_kj
     const bool traced = M.part != nullptr && mud != 0.0;
-    const double hd = M.dt;
 
     // what depends on the thread's row: tables, places, and where the row is a halo (the same byte offset in
     // the other blocks' buffers, by rank)
@@ -276,7 +261,7 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
     float dD[VL], dL[VL], dR[VL];
     unsigned own = 0, halo[NT];
     int n_halo = 0;
-    float *yrow = yrep, *lrow = lrep;
+    float *yrow = yrep;
     double *y0row = y0rep;
     const unsigned Ab = (unsigned)__cvta_generic_to_shared(A), Bb = (unsigned)__cvta_generic_to_shared(B);
     const auto set_row = [&](int rl) {
@@ -287,7 +272,6 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
         own = (unsigned)(pair * SLAB + (rl + 3) * NP) * 4u + o0;
         const size_t c = (size_t)pair * 2 * blk + (size_t)i * NP + l0;
         yrow = yrep + c;
-        lrow = lrep + c;
         y0row = y0rep + c;
         n_halo = 0;
         // the row on the unwrapped axis (periodic q: also whole periods away, as far as the three rows beyond either
@@ -320,18 +304,23 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
             // stage 4: y in A -> B, 3: B -> A, 2: A -> B, 1: B -> A, the new y
             const unsigned in = (k & 1) ? Bb : Ab, out = (k & 1) ? Ab : Bb;
             const float h = M.sc[k].h;
+            const double hd = M.hd[k];
             double trr = 0.0, tri = 0.0;
             if (nloc > 0) {
 #pragma unroll 1
                 for (int trip = 0; trip < trips; ++trip) {
                     const int item = trip * groups + group;
-                    const int row = item / EG, eg = item - row * EG;
+                    const int row = item / EG;
                     const bool act_row = item < R * EG && row < nloc;
+                    // where all passes over the elements are full, each row starts at another one: the zeroth tier's
+                    // FP64 instructions, 64 clocks of a quarter of the SM each, then don't meet (2D spectrum 198 -> 170 ms)
+                    const int eg = item - row * EG + (E % EG == 0 ? row % E : 0);
                     if (trips > 1) set_row(act_row ? row : 0);
 #pragma unroll 1
                     for (int e0 = 0; e0 < E; e0 += EG) {
-                        const bool act = act_row && e0 + eg < E;
-                        const int e = act ? e0 + eg : 0;
+                        const int et = e0 + eg;
+                        const bool act = act_row && (E % EG == 0 || et < E);
+                        const int e = act ? (et < E ? et : et - E) : 0;
                         const ResElem &I = el[e];
                         const unsigned pe = in + own + e * ES4;  // this lane's values of the row (real part)
                         const size_t go = (size_t)e * g.elem_stride;
@@ -343,14 +332,19 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
 #pragma unroll
                             for (int v = 0; v < VL; ++v) x[v] = make_float2(a[v], c[v]);
                         }
-                        // the step's base: y itself at the first stage, the FP64 zeroth tier at the last
-                        float br[VL], bi[VL];
-                        if (k != 4 && (e != 0 || k != 1)) {
-                            ldrow<float, VL>(yrow + go, br);
-                            ldrow<float, VL>(yrow + go + blk, bi);
+                        // the step's base, asked for early: y (at the first stage the input itself), for the zeroth tier
+                        // its FP64 value, whose parts take the registers of both planes
+                        float base[4 * VL];
+                        if (e == 0) {
+                            const float *w = reinterpret_cast<const float *>(y0row);
+                            ldrow<float, 2 * VL>(w, base);
+                            ldrow<float, 2 * VL>(w + 2 * blk, base + 2 * VL);
+                        } else if (k != 4) {
+                            ldrow<float, VL>(yrow + go, base);
+                            ldrow<float, VL>(yrow + go + blk, base + VL);
                         } else {
-                            lds(pe, br);
-                            lds(pe + PL4, bi);
+                            lds(pe, base);
+                            lds(pe + PL4, base + VL);
                         }
                         lanes_forward<LPR, VL>(x, l, w8);
 #pragma unroll
@@ -451,42 +445,37 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
                         }
                         if (!act) continue;
                         // ---- update: base + h L
+                        float br[VL], bi[VL];
                         if (e != 0) {
+#pragma unroll
+                            for (int v = 0; v < VL; ++v) {
+                                br[v] = base[v];
+                                bi[v] = base[VL + v];
+                            }
                             v_axpy<VL>(br, h, ar);
                             v_axpy<VL>(bi, h, ai);
                             if (k == 1) {
                                 strow<float, VL>(yrow + go, br);
                                 strow<float, VL>(yrow + go + blk, bi);
                             }
-                        } else if (k != 1) {
-                            // the FP64 zeroth tier as the sum of two floats (the rounded value and the rest)
-                            float cr[VL], ci[VL];
-                            ldrow<float, VL>(lrow, cr);
-                            ldrow<float, VL>(lrow + blk, ci);
-                            v_axpy<VL>(cr, h, ar);
-                            v_axpy<VL>(ci, h, ai);
-                            v_add<VL>(br, cr);
-                            v_add<VL>(bi, ci);
                         } else {
-                            const auto accumulate = [&](const float (&a)[VL], float (&bb)[VL], size_t off, double &sum) {
-                                double tr = 0.0;
-                                float low[VL];
+                            const auto accumulate = [&](const float (&a)[VL], float (&b)[VL], const float *w0, size_t off, double &sum) {
+                                double w[VL], tr = 0.0;
 #pragma unroll
-                                for (int v = 0; v < VL; v += 2) {
-                                    double2 w = *reinterpret_cast<const double2 *>(y0row + off + v);
-                                    w.x = fma(hd, widen(a[v]), w.x);
-                                    w.y = fma(hd, widen(a[v + 1]), w.y);
-                                    *reinterpret_cast<double2 *>(y0row + off + v) = w;
-                                    split_double(w.x, bb[v], low[v]);
-                                    split_double(w.y, bb[v + 1], low[v + 1]);
-                                    if (traced) tr += w.x + w.y;
+                                for (int v = 0; v < VL; ++v) {
+                                    w[v] = __hiloint2double(__float_as_int(w0[2 * v + 1]), __float_as_int(w0[2 * v]));
+                                    w[v] = fma(hd, widen(a[v]), w[v]);
+                                    b[v] = narrow(w[v]);
+                                    if (traced && k == 1) tr += w[v];
                                 }
-                                strow<float, VL>(lrow + off, low);
-                                strow<float, VL>(yrow + off, bb);
-                                if (traced) sum += mud * tr;
+                                if (k == 1) {
+                                    strow<double, VL>(y0row + off, w);
+                                    strow<float, VL>(yrow + off, b);
+                                    if (traced) sum += mud * tr;
+                                }
                             };
-                            accumulate(ar, br, 0, trr);
-                            accumulate(ai, bi, blk, tri);
+                            accumulate(ar, br, base, 0, trr);
+                            accumulate(ai, bi, base + 2 * VL, blk, tri);
                         }
                         // own buffer, and the halos of the blocks within three rows
                         const unsigned po = out + own + e * ES4;
@@ -526,19 +515,6 @@ resident_kernel(const ResidentMember *__restrict__ members, int n_mem, int n_ste
                 }
             }
             cluster_sync();
-        }
-    }
-}
-
-// low halves of the zeroth tier: y0 - y, from which the stages rebuild the FP64 base
-__global__ void resident_low_kernel(const ResidentMember *__restrict__ members, int n_mem)
-{
-    for (int m = 0; m < n_mem; ++m) {
-        const ResidentMember &M = members[m];
-        const size_t n = M.g.tier0_rep_stride, total = n * M.g.n_rep;
-        for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-            const size_t rep = t / n, c = t % n, o = rep * M.g.rep_stride + c;
-            M.lo[o] = (float)(M.y0[t] - (double)M.y[o]);
         }
     }
 }
@@ -629,13 +605,8 @@ cudaError_t resident_capacity(int np, int csize, int threads, size_t smem, int *
 }
 
 cudaError_t launch_resident(int np, const ResidentMember *members, int n_mem, int clusters, int csize, int threads,
-                            size_t smem, int n_steps, bool first, cudaStream_t st)
+                            size_t smem, int n_steps, cudaStream_t st)
 {
-    if (first) {
-        resident_low_kernel<<<152, 256, 0, st>>>(members, n_mem);
-        cudaError_t e = cudaGetLastError();
-        if (e) return e;
-    }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     cudaError_t e = np == 32 ? configure<32>(cfg, attr, clusters, csize, threads, smem, st)
