@@ -13,8 +13,8 @@
 // Magnitudes (complex): a radix-16 pass takes inputs below 2^60 and scales by 1/4 between its two layers
 // of length-4 transforms (outputs below 2^62); a radix-8 pass takes inputs below 2^59; a twiddle product
 // takes inputs below 2^62 and scales by 1/4 or 1/8.  Every intermediate stays below 2^63.
-// Infinities, NaN and values from 2^1007 (whose sums may overflow): every output of their transform is NaN.
-// Inputs below 2^-1022 count as zero (rows whose largest value is below 2^-958 lose bits).
+// Common exponents of transforms go past those of doubles; conversions near the ends of the range of doubles are
+// to_fixed_any and from_fixed_any.  A row with an infinity or a NaN (exponent EXP_BAD) gives NaN.
 #pragma once
 #include <stdint.h>
 #include <string.h>
@@ -31,7 +31,11 @@ struct I2 {  // complex fixed-point value
     long long x, y;
 };
 
-constexpr int EXP_BIG = 2030;  // common exponents from here on (values from 2^1007, infinities, NaN) give NaN
+// common exponents of a transform: from here on an infinity or a NaN among its inputs
+constexpr int EXP_BAD = 16000;
+// exponents of doubles outside of these (values below 2^-895, from 2^1007) take the functions for any value
+constexpr int EXP_SMALL = 128, EXP_BIG = 2030;
+QH_HD bool exp_plain(int E) { return (unsigned)(E - EXP_SMALL) < (unsigned)(EXP_BIG - EXP_SMALL); }
 
 QH_HD unsigned long long dbits(double v)
 {
@@ -95,6 +99,16 @@ template <int B> QH_HD long long to_fixed(double v, int E)
     return ((long long)m ^ s) - s;
 }
 
+// ... for any E from max(its exponent, 1) on, subnormal values too
+template <int B> QH_HD long long to_fixed_any(double v, int E)
+{
+    const unsigned long long u = dbits(v);
+    const int ex = (int)(u >> 52) & 2047;
+    const unsigned long long m = shr_u(((u & 0xfffffffffffffull) | (ex ? 0x10000000000000ull : 0)) << (B - 53), E - (ex ? ex : 1));
+    const long long s = (long long)u >> 63;
+    return ((long long)m ^ s) - s;
+}
+
 QH_HD int clz64(unsigned long long u)
 {
 #ifdef __CUDA_ARCH__
@@ -104,8 +118,7 @@ QH_HD int clz64(unsigned long long u)
 #endif
 }
 
-// v * 2^K rounded to a double (half away from zero), for common exponents below EXP_BIG (the result is then a
-// normal number).  Integer operations: the conversion instruction takes two and more slots of the FP64
+// v * 2^K rounded to a double (half away from zero), where the result is zero or a normal number.  Integer operations: the conversion instruction takes two and more slots of the FP64
 // pipe (stage on 96 x 128, depth 8: 0.73 ms with it).
 QH_HD double from_fixed(long long v, int K)
 {
@@ -117,6 +130,17 @@ QH_HD double from_fixed(long long v, int K)
     r += (unsigned long long)(unsigned)(K - n + 63 + 1022) << 52;  // the leading bit carries into the exponent
     r |= (unsigned long long)s & 0x8000000000000000ull;
     return bitsd(v ? r : 0);
+}
+
+// v * 2^K over the whole range of doubles: subnormal results and infinities too
+QH_HD double from_fixed_any(long long v, int K)
+{
+    const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
+    const int e = K + 63 - clz64(m) + 1022;
+    if (v == 0 || (unsigned)e <= 2045u) return from_fixed(v, K);
+    K = K < -2044 ? -2044 : (K > 2044 ? 2044 : K);
+    const int h = K >> 1;  // in two steps, the first of them exact
+    return (double)v * bitsd((unsigned long long)(h + 1023) << 52) * bitsd((unsigned long long)(K - h + 1023) << 52);
 }
 
 // The two halves of a 64-bit factor, the low one signed: c = h * 2^32 + l

@@ -467,6 +467,9 @@ template <int NP> struct FixedRows {
     }
 };
 
+// (a function of its own: few rows need it)
+template <int B> __device__ __noinline__ long long far_fixed(double v, int E) { return qhfx::to_fixed_any<B>(v, E); }
+
 // rows * S2 p-rows of the tile into X as integers below 2^bits of their row's exponent
 template <int NP, int S2>
 __device__ __forceinline__ void fill_fixed(double2 *X, const double *__restrict__ v, size_t blk, int i0, int rows)
@@ -485,14 +488,21 @@ __device__ __forceinline__ void fill_fixed(double2 *X, const double *__restrict_
         double re[LV], im[LV];
         ldrow<double, LV>(src, re);
         ldrow<double, LV>(src + blk, im);
-        int E = common_exponent<LV>(re, im);
+        int E = 1;
+#pragma unroll
+        for (int q = 0; q < LV; ++q) E = max(E, max(exponent_of(re[q]), exponent_of(im[q])));
 #pragma unroll
         for (int o = PL / 2; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
         if (act) {
             I2 *x = reinterpret_cast<I2 *>(X + pad16(rp * NP + l));
+            if (E >= EXP_SMALL) {
 #pragma unroll
-            for (int q = 0; q < LV; ++q) x[q] = I2{to_fixed<B>(re[q], E), to_fixed<B>(im[q], E)};
-            if (l == 0) F::exp_slot(X, rp, F::FWD_EXP) = (short)E;
+                for (int q = 0; q < LV; ++q) x[q] = I2{to_fixed<B>(re[q], E), to_fixed<B>(im[q], E)};
+            } else {
+#pragma unroll
+                for (int q = 0; q < LV; ++q) x[q] = I2{dbits(re[q]) << 1 ? far_fixed<B>(re[q], E) : 0, dbits(im[q]) << 1 ? far_fixed<B>(im[q], E) : 0};
+            }
+            if (l == 0) F::exp_slot(X, rp, F::FWD_EXP) = (short)(E < 2047 ? E : EXP_BAD);
         }
     }
 }
@@ -517,8 +527,8 @@ template <int NP> __device__ __noinline__ void pass16_fixed(double2 *X, int n_tr
 
 template <int NP, int S>
 __device__ __forceinline__ void potential_fixed(double2 *X, const double2 *tw, const FusedTables<double> &tab, int nq, int i0,
-                                                int rows, double fpp, double ngam, const double *s_lpp, double c2,
-                                                double q_min, double dq)
+                                                int rows, double fpp, double ngam, const double *s_lpp, int &s_far,
+                                                double c2, double q_min, double dq)
 {
     using namespace qhfx;
     using F = FixedRows<NP>;
@@ -606,7 +616,6 @@ __device__ __forceinline__ void potential_fixed(double2 *X, const double2 *tw, c
                     if (s != j_) M = max(M, E[s * S + k] + kL[(j_ * S + s) * nq + i]);
                     if (s != k) M = max(M, E[j_ * S + s] + kR[(s * S + k) * nq + i]);
                 }
-                M = max(M, 100);
                 long long ar[MV], ai[MV];  // the commutator: at most six products below 2^60
                 {
                     const int sh = M - (E[jk] + kD[jk * nq + i]);
@@ -649,7 +658,7 @@ __device__ __forceinline__ void potential_fixed(double2 *X, const double2 *tw, c
                 const int n = norm_shift<59>(__reduce_or_sync(run, o));
 #pragma unroll
                 for (int v = 0; v < MV; ++v) XI[tr * PNP + pad16(pos0 + v)] = shift(q[v], n);
-                if (pos0 % 16 == 0) F::exp_slot(X, tr, pos0 / 16) = (short)(big >= EXP_BIG ? EXP_BIG : min(M - n, EXP_BIG));
+                if (pos0 % 16 == 0) F::exp_slot(X, tr, pos0 / 16) = (short)(big >= EXP_BAD ? EXP_BAD : M - n);
             }
     }
     __syncthreads();
@@ -668,11 +677,14 @@ __device__ __forceinline__ void potential_fixed(double2 *X, const double2 *tw, c
         inverse_butterfly<R0>(x, w62, j);
 #pragma unroll
         for (int t = 0; t < R0; ++t) xb[17 * t] = I2{x[t].y, x[t].x};
-        if (j == 0) F::exp_slot(X, tr, F::FWD_EXP) = (short)E;
+        if (j == 0) {
+            F::exp_slot(X, tr, F::FWD_EXP) = (short)E;
+            if (!exp_plain(E)) s_far = 1;
+        }
     }
     __syncthreads();
 }
-// the potential term in X is v 2^(E + fixed_pot_exponent), E at the transform's FWD_EXP (EXP_BIG: NaN)
+// the potential term in X is v 2^(E + fixed_pot_exponent), E at the transform's FWD_EXP (EXP_BAD: NaN)
 template <int NP, int S> constexpr int fixed_pot_exponent()
 {
     constexpr int R0 = Radices<NP>::r[0];
@@ -687,7 +699,7 @@ template <int NP, int S> __device__ __forceinline__ void potential_to_double(dou
         const I2 v = reinterpret_cast<const I2 *>(X)[pad16(t)];
         const double bad = bitsd(0x7ff8000000000000ull);
         const int K = M + fixed_pot_exponent<NP, S>();
-        X[pad16(t)] = M >= EXP_BIG ? double2{bad, bad} : double2{from_fixed(v.x, K), from_fixed(v.y, K)};
+        X[pad16(t)] = M >= EXP_BAD ? double2{bad, bad} : double2{from_fixed_any(v.x, K), from_fixed_any(v.y, K)};
     }
 }
 
@@ -702,6 +714,56 @@ __device__ __forceinline__ FixedWeight fixed_weight(double w)
     if (ex == 0) return FixedWeight{{0, 0}, -4096};  // far below every other term
     const long long m = qhfx::to_fixed<62>(w, ex);
     return FixedWeight{qhfx::halves(m), ex - 1022};
+}
+
+// weight of the t-th of the six rows of the upwind q difference
+__device__ __forceinline__ int upwind_weight(bool neg, int t)
+{
+    const int s = neg ? 5 - t : t;
+    const int w = s == 0 ? -2 : s == 1 ? 15 : s == 2 ? -60 : s == 3 ? 20 : s == 4 ? 30 : -3;
+    return neg ? -w : w;
+}
+
+// A value's q difference times pk, in FP64, and its potential term pot 2^K: the column V, window rows from ii on
+__device__ __noinline__ double far_value(const double *V, int np, int ii, int nq, int periodic, bool neg, double pk,
+                                         long long pot, int K)
+{
+    double kin = 0.0;
+#pragma unroll 1
+    for (int t = 0; t < 6; ++t) {
+        int i = ii + t;
+        const bool ok = i >= 0 && i < nq;
+        if (!ok && periodic) i = wrap_q(i, nq);
+        kin = fma((double)upwind_weight(neg, t), ok || periodic ? V[(size_t)i * np] : 0.0, kin);
+    }
+    return fma(pk, kin, qhfx::from_fixed_any(pot, K));
+}
+
+template <int VEC> __device__ __forceinline__ bool nonzero(const double *x)
+{
+    unsigned long long any = 0;
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) any |= qhfx::dbits(x[v]) << 1;
+    return any != 0;
+}
+
+// e: a p row's values x with two on each side (periodic p), a warp a row
+template <int VEC, typename T> __device__ __forceinline__ void with_neighbours(const T *x, T *e, int lane)
+{
+    const unsigned all = 0xffffffffu;
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) e[v + 2] = x[v];
+    if constexpr (VEC == 1) {
+        e[0] = __shfl_sync(all, x[0], (lane + 30) & 31);
+        e[1] = __shfl_sync(all, x[0], (lane + 31) & 31);
+        e[3] = __shfl_sync(all, x[0], (lane + 1) & 31);
+        e[4] = __shfl_sync(all, x[0], (lane + 2) & 31);
+    } else {
+        e[0] = __shfl_sync(all, x[VEC - 2], (lane + 31) & 31);
+        e[1] = __shfl_sync(all, x[VEC - 1], (lane + 31) & 31);
+        e[VEC + 2] = __shfl_sync(all, x[0], (lane + 1) & 31);
+        e[VEC + 3] = __shfl_sync(all, x[1], (lane + 1) & 31);
+    }
 }
 
 // Phase B of the FP64 form (linear coupling, all terms, the potential and the p-diagonal bath terms already
@@ -719,12 +781,13 @@ __device__ __forceinline__ FixedWeight fixed_weight(double w)
 //            to the largest exponent, 57 bits below it, and the p difference (weights 1, 8) is exact.
 // Quantising at 2^-54 to 2^-62 of the largest term is below the rounding of the FP64 sums, whose partial sums of
 // up to 100 times the values round at 2^-53.
-// Infinities, NaN and values from 2^1007: a column or row that holds one gives NaN.
+// Rows whose differences or potential term are near the ends of the range of doubles (exp_plain) have their q differences
+// in FP64, values by value, and so do the p differences of such rows: subnormal values, infinities and NaN as in FP64 sums.
 template <int NP, int S>
 __device__ __forceinline__ void
 rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__restrict__ v_in, const double *y, double *v_out,
            int mode, size_t ebase, int i0, int rows, const long long *nb_off, const double *nb_wg, const double *nb_wa,
-           int n_up, int n_d0, int n_nb, bool term, double2 *X, const double *pgrid)
+           int n_d0, int n_nb, bool term, bool any_far, double2 *X, const double *pgrid)
 {
     using namespace qhfx;
     constexpr int S2 = S * S;
@@ -737,11 +800,8 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
     const int l0 = lane * VEC;
     const bool neg = pgrid[l0] < 0.0;  // one sign per lane (caller's check)
     int ck[6];                         // p < 0: offsets -2..+3, p >= 0: -3..+2
-    {
-        const int cneg[6] = {3, -30, -20, 60, -15, 2}, cpos[6] = {-2, 15, -60, 20, 30, -3};
 #pragma unroll
-        for (int t = 0; t < 6; ++t) ck[t] = neg ? cneg[t] : cpos[t];
-    }
+    for (int t = 0; t < 6; ++t) ck[t] = upwind_weight(neg, t);
     const int first = neg ? -2 : -3;
     const double bad = bitsd(0x7ff8000000000000ull);
     int rg = min(RG, (rows * S2 + FTHREADS / 32 - 1) / (FTHREADS / 32));  // fewer where warps would idle
@@ -754,6 +814,14 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
         const int nr = min(us + rg, i0 + rows) - ia;
         const int gs = ia & ~(RG - 1), k0 = ia - gs;  // the group of RG grid rows that the unit's are among
         const size_t poff = ebase + (size_t)pr * 2 * blk;
+        // the unit's rows in the group, by the exponent of their potential term
+        unsigned near = ((1u << nr) - 1) << k0, far = 0;
+        if (any_far) {
+#pragma unroll 1
+            for (int r = 0; r < nr; ++r)
+                if (!exp_plain(FixedRows<NP>::exp_slot(X, (r0 + r) * S2 + pr, FixedRows<NP>::FWD_EXP))) far |= 1u << (k0 + r);
+            near &= ~far;
+        }
 #pragma unroll 1
         for (int plane = 0; plane < 2; ++plane) {
             const double *V = v_in + poff + plane * blk;
@@ -776,6 +844,9 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                 // row r from its six window rows x (below 2^62) of exponent E: -p dW/dq and the potential term, each
                 // an integer, at the larger unit
                 const auto emit = [&](int r, const Half *x, int E) {
+                    double &xv = Xat(r, v);
+                    const long long pot = (long long)dbits(xv);
+                    const int M = FixedRows<NP>::exp_slot(X, (r0 + r) * S2 + pr, FixedRows<NP>::FWD_EXP);
                     long long lo = 0, hi = 0;
 #pragma unroll
                     for (int t = 0; t < 6; ++t) {
@@ -783,14 +854,10 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                         hi = madw(x[t].h, ck[t], hi);
                     }
                     const long long kin = mul_hi(halves((long long)((unsigned long long)hi << 24) + (lo >> 8)), pk.c);
-                    double &xv = Xat(r, v);
-                    const long long pot = (long long)dbits(xv);
-                    const int M = FixedRows<NP>::exp_slot(X, (r0 + r) * S2 + pr, FixedRows<NP>::FWD_EXP);
                     const int uk = E + pk.k - 1022 - 62 + 8 + 2, up = M + fixed_pot_exponent<NP, S>();
-                    const int U = max(max(uk, up), -1000);  // (below 2^60 and 2^62: the sum fits)
+                    const int U = max(uk, up);  // (below 2^60 and 2^62: the sum fits)
                     const long long fine = uk < up ? kin : pot, coarse = uk < up ? pot : kin;
-                    const double a = from_fixed(shr_round(coarse, U - max(uk, up)) + shr_round(fine, U - min(uk, up)), U);
-                    xv = E >= EXP_BIG || M >= EXP_BIG ? bad : a;
+                    xv = from_fixed(coarse + shr_round(fine, U - min(uk, up)), U);
                 };
                 double raw[RG + 5];
                 int ex[RG + 5], E = EXP_MIN;
@@ -807,6 +874,15 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                     const int er = max(max(max(ex[r], ex[r + 1]), max(ex[r + 2], ex[r + 3])), max(ex[r + 4], ex[r + 5]));
                     if (gs + r < nq) least = min(least, er);
                 }
+                unsigned odd = far;  // rows left to FP64
+                bool zero = false;  // nothing but zeros in the window
+                if (!exp_plain(E)) {
+                    unsigned long long any = 0;
+#pragma unroll
+                    for (int t = 0; t < RG + 5; ++t) any |= dbits(raw[t]) << 1;
+                    zero = any == 0;
+                    if (!zero) least = -EXP_BIG;  // each row by itself
+                }
                 if (!__any_sync(0xffffffffu, E - least > 8)) {
                     Half x[RG + 5];
 #pragma unroll
@@ -814,19 +890,31 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                         x[t] = halves(to_fixed<62>(raw[t], E));
 #pragma unroll
                     for (int r = 0; r < RG; ++r)
-                        if (r >= k0 && r < k0 + nr) emit(r - k0, x + r, E);
+                        if (near >> r & 1) emit(r - k0, x + r, E);
                 } else {  // steep in q: an exponent for each row
 #pragma unroll
                     for (int r = 0; r < RG; ++r) {
-                        if (r < k0 || r >= k0 + nr) continue;
+                        if (!(near >> r & 1)) continue;
                         int er = EXP_MIN;
 #pragma unroll
                         for (int t = 0; t < 6; ++t) er = max(er, ex[r + t]);
                         Half x[6];
 #pragma unroll
                         for (int t = 0; t < 6; ++t) x[t] = halves(to_fixed<62>(raw[r + t], er));
-                        emit(r - k0, x, er);
+                        if (exp_plain(er) || zero) emit(r - k0, x, er);
+                        else odd |= 1u << r;
                     }
+                }
+#pragma unroll 1
+                for (int r = -k0; odd; ++r, odd >>= 1) {
+                    if (!(odd & 1)) continue;
+                    double &xv = Xat(r, v);
+                    const int M = FixedRows<NP>::exp_slot(X, (r0 + r) * S2 + pr, FixedRows<NP>::FWD_EXP);
+                    if (zero && dbits(xv) == 0 && M < EXP_BAD) continue;  // (a zero as an integer and as a double)
+                    xv = M >= EXP_BAD ? bad
+                                      : far_value(V + l0 + v, NP, gs + first + k0 + r, nq, g.periodic_q, neg,
+                                                  -(pgrid[l0 + v] * sc.fkin), (long long)dbits(xv),
+                                                  M + fixed_pot_exponent<NP, S>());
                 }
             }
             double p[VEC], pw[VEC];  // p, and times the weight of the (first) neighbour with a p term
@@ -880,30 +968,22 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
 #pragma unroll
                     for (int v = 0; v < VEC; ++v) E = max(E, exponent_of(G[v]));
                     E = __reduce_max_sync(0xffffffffu, E);
-                    long long Gi[VEC];
+                    if (exp_plain(E)) {
+                        long long Gi[VEC], e[VEC + 4];
 #pragma unroll
-                    for (int v = 0; v < VEC; ++v) Gi[v] = to_fixed<BITS>(G[v], E);
-                    long long e[VEC + 4];
+                        for (int v = 0; v < VEC; ++v) Gi[v] = to_fixed<BITS>(G[v], E);
+                        with_neighbours<VEC>(Gi, e, lane);
 #pragma unroll
-                    for (int v = 0; v < VEC; ++v) e[v + 2] = Gi[v];
-                    const unsigned all = 0xffffffffu;
-                    if constexpr (VEC == 1) {
-                        e[0] = __shfl_sync(all, Gi[0], (lane + 30) & 31);
-                        e[1] = __shfl_sync(all, Gi[0], (lane + 31) & 31);
-                        e[3] = __shfl_sync(all, Gi[0], (lane + 1) & 31);
-                        e[4] = __shfl_sync(all, Gi[0], (lane + 2) & 31);
-                    } else {
-                        e[0] = __shfl_sync(all, Gi[VEC - 2], (lane + 31) & 31);
-                        e[1] = __shfl_sync(all, Gi[VEC - 1], (lane + 31) & 31);
-                        e[VEC + 2] = __shfl_sync(all, Gi[0], (lane + 1) & 31);
-                        e[VEC + 3] = __shfl_sync(all, Gi[1], (lane + 1) & 31);
-                    }
+                        for (int v = 0; v < VEC; ++v) {
+                            const long long d = (e[v] - e[v + 4]) + ((e[v + 3] - e[v + 1]) << 3);
+                            a[v] = fma(sc.inv12dp, from_fixed(d, E - 1022 - BITS), a[v]);
+                        }
+                    } else if (__any_sync(0xffffffffu, nonzero<VEC>(G))) {  // (warp-uniform)
+                        double e[VEC + 4];
+                        with_neighbours<VEC>(G, e, lane);
 #pragma unroll
-                    for (int v = 0; v < VEC; ++v) {
-                        const long long d = (e[v] - e[v + 4]) + ((e[v + 3] - e[v + 1]) << 3);
-                        double dg = from_fixed(d, E - 1022 - BITS);
-                        if (E >= EXP_BIG) dg = bad;
-                        a[v] = fma(sc.inv12dp, dg, a[v]);
+                        for (int v = 0; v < VEC; ++v)
+                            a[v] = fma(sc.inv12dp, e[v] - 8.0 * e[v + 1] + 8.0 * e[v + 3] - e[v + 4], a[v]);
                     }
                 }
                 if (mode != 0) {
@@ -1155,6 +1235,7 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
     __shared__ long long mx_off[QH_MAX_MODES];  // nonlinear coupling: mixed-derivative neighbours
     __shared__ T mx_w[QH_MAX_MODES];
     __shared__ int s_nmx;
+    __shared__ int s_far;  // FP64: a row whose potential term's exponent is not plain
     __shared__ int s_cnt[4];
     __shared__ T s_ngam;
     __shared__ __align__(16) T pgrid[NP];
@@ -1192,6 +1273,7 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
             mx_w[a] = (T)(E.wmx[a] / (12.0 * g.dq));
         }
         s_nmx = n_mx;
+        s_far = 0;
         s_cnt[0] = n_up;
         s_cnt[2] = n;
         s_cnt[3] = (terms & 8) && E.terminator;
@@ -1220,7 +1302,7 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
             __syncthreads();
             potential_fixed<NP, S>(X, tw, tab, nq, i0, rows,
                                    ((terms & 4) ? sc.fdelta : (T)0) + ((s_cnt[3] != 0) ? sc.fterm : (T)0), s_ngam, s_lpp,
-                                   NL ? g.c2 : 0.0, g.q_min, g.dq);
+                                   s_far, NL ? g.c2 : 0.0, g.q_min, g.dq);
         }
     } else if (fold) {
         constexpr int LV = 4;  // p values per load
@@ -1265,8 +1347,8 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
         // the fixed-point form: all terms, the potential in X, every lane's p values of one sign
         const bool one_sign = __all_sync(0xffffffffu, (pgrid[lane * (NP / 32)] < (T)0) == (pgrid[lane * (NP / 32) + NP / 32 - 1] < (T)0));
         if (fold && terms == QHFPE_TERM_ALL && one_sign) {
-            rows_fixed<NP, S>(g, sc, v_in, y, v_out, mode, ebase, i0, rows, nb_off, nb_wg, nb_wa, n_up, n_d0, n_nb, term, X,
-                              pgrid);
+            rows_fixed<NP, S>(g, sc, v_in, y, v_out, mode, ebase, i0, rows, nb_off, nb_wg, nb_wa, n_d0, n_nb, term,
+                              s_far != 0, X, pgrid);
             return;
         }
     }
