@@ -608,7 +608,7 @@ qhfpe_status build_model(qhfpe *h, Model &M, int S, const double *U, const doubl
         for (size_t r = 0; r < n_rows; ++r) {
             double *row = ft.data() + r * p.np, big = 0.0;
             for (int t = 0; t < p.np; ++t) big = std::max(big, std::fabs(row[t]));
-            int k = -4096;  // a row of zeros: below every other term
+            int k = -4096;  // a row of zeros (EXP_NO_TABLE): below every other term
             if (big > 0.0) std::frexp(big, &k);
             kx[r] = k;
             const bool plain = std::abs(k) < 900;  // 2^(62 - k) is a normal double: the product is exact

@@ -488,19 +488,27 @@ __device__ __forceinline__ void fill_fixed(double2 *X, const double *__restrict_
         double re[LV], im[LV];
         ldrow<double, LV>(src, re);
         ldrow<double, LV>(src + blk, im);
-        int E = 1;
+        unsigned top = 0, low = 0;  // the row's largest upper half; zero for a row of zeros only
 #pragma unroll
-        for (int q = 0; q < LV; ++q) E = max(E, max(exponent_of(re[q]), exponent_of(im[q])));
+        for (int q = 0; q < LV; ++q) {
+            top = max(top, max((unsigned)__double2hiint(re[q]) & 0x7fffffffu, (unsigned)__double2hiint(im[q]) & 0x7fffffffu));
+            low |= (unsigned)__double2loint(re[q]) | (unsigned)__double2loint(im[q]);
+        }
+        top |= low != 0u;
 #pragma unroll
-        for (int o = PL / 2; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+        for (int o = PL / 2; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+        const int E = top >= 0x00100000u ? (int)(top >> 20) : (top ? 1 : EXP_NONE);
         if (act) {
             I2 *x = reinterpret_cast<I2 *>(X + pad16(rp * NP + l));
             if (E >= EXP_SMALL) {
 #pragma unroll
                 for (int q = 0; q < LV; ++q) x[q] = I2{to_fixed<B>(re[q], E), to_fixed<B>(im[q], E)};
+            } else if (E == EXP_NONE) {
+#pragma unroll
+                for (int q = 0; q < LV; ++q) x[q] = I2{0, 0};
             } else {
 #pragma unroll
-                for (int q = 0; q < LV; ++q) x[q] = I2{dbits(re[q]) << 1 ? far_fixed<B>(re[q], E) : 0, dbits(im[q]) << 1 ? far_fixed<B>(im[q], E) : 0};
+                for (int q = 0; q < LV; ++q) x[q] = I2{far_fixed<B>(re[q], E), far_fixed<B>(im[q], E)};
             }
             if (l == 0) F::exp_slot(X, rp, F::FWD_EXP) = (short)(E < 2047 ? E : EXP_BAD);
         }
@@ -569,7 +577,7 @@ __device__ __forceinline__ void potential_fixed(double2 *X, const double2 *tw, c
     const auto bath = [&](double f) {
         const double bound = (64.0 * fabs(f) + fabs(ngam)) * (1.0 / NP);
         const int Eb = max(exponent_of(bound) + 1, EXP_MIN);
-        kcf = bound > 0.0 ? Eb - 1022 : -4096;
+        kcf = bound > 0.0 ? Eb - 1022 : EXP_NO_TABLE;
 #pragma unroll
         for (int v = 0; v < MV; ++v) cf[v] = halves(to_fixed<62>(f * s_lpp[pos0 + v] - ngam * (1.0 / NP), Eb));
     };
@@ -679,7 +687,7 @@ __device__ __forceinline__ void potential_fixed(double2 *X, const double2 *tw, c
         for (int t = 0; t < R0; ++t) xb[17 * t] = I2{x[t].y, x[t].x};
         if (j == 0) {
             F::exp_slot(X, tr, F::FWD_EXP) = (short)E;
-            if (!exp_plain(E)) s_far = 1;
+            if (exp_far(E)) s_far = 1;
         }
     }
     __syncthreads();
@@ -819,7 +827,7 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
         if (any_far) {
 #pragma unroll 1
             for (int r = 0; r < nr; ++r)
-                if (!exp_plain(FixedRows<NP>::exp_slot(X, (r0 + r) * S2 + pr, FixedRows<NP>::FWD_EXP))) far |= 1u << (k0 + r);
+                if (exp_far(FixedRows<NP>::exp_slot(X, (r0 + r) * S2 + pr, FixedRows<NP>::FWD_EXP))) far |= 1u << (k0 + r);
             near &= ~far;
         }
 #pragma unroll 1
@@ -910,7 +918,6 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
                     if (!(odd & 1)) continue;
                     double &xv = Xat(r, v);
                     const int M = FixedRows<NP>::exp_slot(X, (r0 + r) * S2 + pr, FixedRows<NP>::FWD_EXP);
-                    if (zero && dbits(xv) == 0 && M < EXP_BAD) continue;  // (a zero as an integer and as a double)
                     xv = M >= EXP_BAD ? bad
                                       : far_value(V + l0 + v, NP, gs + first + k0 + r, nq, g.periodic_q, neg,
                                                   -(pgrid[l0 + v] * sc.fkin), (long long)dbits(xv),
@@ -1235,7 +1242,7 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
     __shared__ long long mx_off[QH_MAX_MODES];  // nonlinear coupling: mixed-derivative neighbours
     __shared__ T mx_w[QH_MAX_MODES];
     __shared__ int s_nmx;
-    __shared__ int s_far;  // FP64: a row whose potential term's exponent is not plain
+    __shared__ int s_far;  // FP64: a row whose potential term's exponent is far from doubles'
     __shared__ int s_cnt[4];
     __shared__ T s_ngam;
     __shared__ __align__(16) T pgrid[NP];
