@@ -363,9 +363,12 @@ __device__ __forceinline__ void strow(T *p, const T *i)
 // three states took 34.4 ms for four steps with four, 35.7 with three, 43.2 with five, which spill).
 // FP64 (integer arithmetic, latency-bound below 16 warps) runs four at 128 registers: on 96 x 128 at depth 8
 // three, four and five blocks took within 3 % of each other, two 25 % longer.
+// Its np 256 spills at four (1200 to 3800 bytes stored, at three 440 to 1140, at two none); us a step with two, three
+// and four blocks: two states, 100 x 256, depth 4 1139, 1105, 1090; 24 x 256, depth 2 158, 178, 213; three states, 80 x
+// 256, depth 4 3081, 3086, 3260; one state, 150 x 256, depth 40 583, 419, 431; c2 != 0, 100 x 256 1781, 1730, 1776.
 template <typename T, int NP, int S>
 struct FusedOcc {
-    static constexpr int blocks = sizeof(T) == 4 ? (NP >= 256 ? 4 : (S >= 3 ? 6 : 7)) : 4;
+    static constexpr int blocks = sizeof(T) == 4 ? (NP >= 256 ? 4 : (S >= 3 ? 6 : 7)) : (NP >= 256 ? 3 : 4);
 };
 
 // Phase A of the fused stage kernels: the potential term of Eq. (quantum-liouvillian) in place on the
