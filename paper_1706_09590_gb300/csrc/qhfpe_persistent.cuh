@@ -139,7 +139,7 @@ __device__ bool trace_step(const GridInfo &g, const TraceJob &tj, long slot, con
 
 // NL: the nonlinear coupling's terms compiled in (the member's c2 != 0).
 template <typename T, int NP, int S, bool MIXED, bool NL>
-__global__ void __launch_bounds__(FTHREADS, FusedOcc<T, NP, S>::blocks - (FusedOcc<T, NP, S>::blocks > 2 ? 1 : 0))
+__global__ void __launch_bounds__(FTHREADS, FusedOcc<T, NP, S>::blocks - (FusedOcc<T, NP, S>::blocks > 3 ? 1 : 0))
 persistent_steps_kernel(const MultiMember<T> *__restrict__ mem, long n_items, int tq, int n_steps, TraceJob tj,
                         GridBarrier bar)
 {
