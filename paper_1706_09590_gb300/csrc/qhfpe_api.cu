@@ -878,6 +878,15 @@ qhfpe_status step_dispatch(qhfpe *h, Prop &P, bool record)
 // times, timed with CUDA events on the handle's stream; the fastest is kept for this propagator.
 // Results do not depend on the tile (every cell is computed by the same arithmetic), only on the form: the q-window kernel
 // adds a cell's FP32 terms in another order than the general one.
+// QHFPE_TILE_ROWS pins the tile (1 .. the limit) instead of timing the candidates, e.g. to profile the launch
+// configuration that a timed run chose.  0: nothing, or no height of this shape.
+int pinned_rows(int limit)
+{
+    const char *env = std::getenv("QHFPE_TILE_ROWS");
+    const int t = env ? std::atoi(env) : 0;
+    return t >= 1 && t <= limit ? t : 0;
+}
+
 qhfpe_status autotune(qhfpe *h, Prop &P)
 {
     const Model &M = *P.m;
@@ -885,14 +894,9 @@ qhfpe_status autotune(qhfpe *h, Prop &P)
     cudaStream_t st = h->stream;
     const int esize = P.mixed ? 4 : 8;
     const int tmax = std::min(fused_max_rows(P.g.np, P.g.S, esize), P.g.nq);
-    // QHFPE_TILE_ROWS pins the tile (1 .. the limit) instead of timing the candidates, e.g. to profile
-    // the launch configuration that a timed run chose
-    if (const char *env = std::getenv("QHFPE_TILE_ROWS")) {
-        const int t = std::atoi(env);
-        if (t >= 1 && t <= tmax) {
-            P.tq = t;
-            return QHFPE_OK;
-        }
+    if (const int t = pinned_rows(tmax)) {
+        P.tq = t;
+        return QHFPE_OK;
     }
     cudaEvent_t a, b;
     QH_CK(h, cudaEventCreate(&a));
@@ -1050,7 +1054,7 @@ qhfpe_status run_persistent(qhfpe *h, Prop &P, long n_steps, double *trace_dev, 
 // ---- resident propagation ------------------------------------------------------------------------
 // Mixed-form two-state propagators with np 32 or 64, linear coupling, no learned closure and the Condon
 // trace, whose lanes' p values share a sign.  QHFPE_RESIDENT=0 keeps the launch-per-stage form, as does
-// QHFPE_TILE_ROWS (which pins that form's tile) and kernel timing (which counts its launches).
+// a valid QHFPE_TILE_ROWS (which pins that form's tile) and kernel timing (which counts its launches).
 bool resident_wanted(const qhfpe *h, const Prop &P)
 {
     const Model &M = *P.m;
@@ -1059,7 +1063,7 @@ bool resident_wanted(const qhfpe *h, const Prop &P)
     for (int c = 0; c < P.g.np; c += 8)  // (a lane has four or eight)
         if (((float)(P.g.p_min + c * P.g.dp) < 0.f) != ((float)(P.g.p_min + (c + 7) * P.g.dp) < 0.f)) return false;
     const char *r = std::getenv("QHFPE_RESIDENT");
-    return !(r && std::strcmp(r, "0") == 0) && !std::getenv("QHFPE_TILE_ROWS");
+    return !(r && std::strcmp(r, "0") == 0) && !pinned_rows(std::min(fused_max_rows(P.g.np, P.g.S, 4), P.g.nq));
 }
 
 // Blocks per cluster: the most (up to 16) with which all clusters run at once, so that few replicas spread
@@ -2524,12 +2528,9 @@ qhfpe_status batch_autotune(qhfpe_batch *b, cudaStream_t st)
     for (qhfpe *h : b->mem) nq_max = std::max(nq_max, h->main->g.nq);
     tmax = std::min(tmax, nq_max);
     auto upload = [&](int tq) { return b->mixed ? batch_upload<float>(b, tq) : batch_upload<double>(b, tq); };
-    if (const char *env = std::getenv("QHFPE_TILE_ROWS")) {
-        const int t = std::atoi(env);
-        if (t >= 1 && t <= tmax) {
-            b->tq = t;
-            return upload(t);
-        }
+    if (const int t = pinned_rows(tmax)) {
+        b->tq = t;
+        return upload(t);
     }
     cudaEvent_t e0, e1;
     QH_CK(h0, cudaEventCreate(&e0));
