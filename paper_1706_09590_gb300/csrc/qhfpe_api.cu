@@ -1936,7 +1936,7 @@ qhfpe_status equilibrium_start(qhfpe_t *h, std::unique_ptr<Prop> &GP)
     Model &G = *h->ground;
     r = make_prop(h, &G, 1, false, p.dt, GP);
     if (r != QHFPE_OK) return r;
-    if (!std::getenv("QHFPE_TILE_ROWS")) {
+    if (!std::getenv("QHFPE_TILE_ROWS")) {  // (a height that the variable holds is taken by the first run)
         GP->tq = G.tuned_tq;
         GP->form = G.tuned_form;
     }
@@ -1993,8 +1993,10 @@ qhfpe_status equilibrium_residual(qhfpe_t *h, Prop &GP, double *res)
 // also written to every replica.
 qhfpe_status equilibrium_embed(qhfpe_t *h, Prop &GP)
 {
-    h->ground->tuned_tq = GP.tq;
-    h->ground->tuned_form = GP.form;
+    if (GP.form >= 0) {  // the autotuner's choice, not a pinned tile
+        h->ground->tuned_tq = GP.tq;
+        h->ground->tuned_form = GP.form;
+    }
     const int S = h->p.n_states;
     const Model &G = *h->ground;
     const size_t blk = (size_t)h->p.nq * h->p.np;
