@@ -1107,20 +1107,54 @@ bool resident_plan(const std::vector<const Prop *> &props, ResidentPlan &R)
     return found;
 }
 
-// (complete on return: the model's next run may be on another stream, a batch's on its first member's)
-qhfpe_status resident_tables(qhfpe *h, Model &M, const double *U, cudaStream_t st)
+// warps of a cluster, each with its part of the trace; doubles of one step's trace parts
+int resident_parts(const ResidentPlan &R) { return R.csize * (R.threads / 32); }
+size_t resident_step_doubles(const ResidentPlan &R) { return (size_t)R.clusters * resident_parts(R) * 2; }
+// steps per launch: bounded so that a launch stays well below a second and the parts below 64 MB
+long resident_steps(const ResidentPlan &R)
 {
-    if (M.rtab) return QHFPE_OK;
-    std::vector<double> t;
-    const int np = M.np;
-    build_tables(M, U, t, [np](int pos) { return resident_frequency(np, pos); }, 0, true);
-    std::vector<float> f(t.begin(), t.end());
-    float *d = nullptr;
-    QH_CK(h, dalloc(&d, f.size()));
-    const cudaError_t e = upload(d, f.data(), f.size() * sizeof(float), st);
-    if (e) cudaFree(d);
-    QH_CK(h, e);
-    M.rtab = d;
+    return std::max<long>(1, std::min<long>(4096, (8l << 20) / (long)resident_step_doubles(R)));
+}
+
+// The device memory that a run takes beside the states: tables, descriptions, trace parts.  *ok = false where it
+// cannot be had; the caller then launches per stage, which needs none of it.
+qhfpe_status resident_prepare(qhfpe *h, const std::vector<Prop *> &props, const std::vector<const double *> &U, bool record,
+                              ResidentPlan &R, long n_steps, cudaStream_t st, bool *ok)
+{
+    const auto have = [&](cudaError_t e) {
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            *ok = false;
+            return cudaSuccess;
+        }
+        return e;
+    };
+    *ok = true;
+    const int np = props[0]->g.np;
+    for (size_t m = 0; m < props.size(); ++m) {
+        Model &M = *props[m]->m;
+        if (M.rtab) continue;
+        // (complete on return: the model's next run may be on another stream, a batch's on its first member's)
+        std::vector<double> t;
+        build_tables(M, U[m], t, [np](int pos) { return resident_frequency(np, pos); }, 0, true);
+        std::vector<float> f(t.begin(), t.end());
+        float *d = nullptr;
+        QH_CK(h, have(dalloc(&d, f.size())));
+        if (!*ok) return QHFPE_OK;
+        const cudaError_t e = upload(d, f.data(), f.size() * sizeof(float), st);
+        if (e) cudaFree(d);
+        QH_CK(h, e);
+        M.rtab = d;
+    }
+    if (!R.desc) QH_CK(h, have(cudaMalloc(&R.desc, props.size() * sizeof(ResidentMember))));
+    const size_t need = record ? resident_step_doubles(R) * (size_t)std::min(resident_steps(R), n_steps) : 0;
+    if (*ok && R.part_cap < need) {
+        if (R.part) cudaFree(R.part);
+        R.part = nullptr;
+        R.part_cap = 0;
+        QH_CK(h, have(dalloc(&R.part, need)));
+        if (*ok) R.part_cap = need;
+    }
     return QHFPE_OK;
 }
 
@@ -1131,21 +1165,8 @@ qhfpe_status run_resident(qhfpe *h, const std::vector<Prop *> &props, const std:
     const int np = props[0]->g.np;
     std::vector<ResidentMember> d(props.size());
     const bool record = !traces.empty();
-    if (!R.desc) QH_CK(h, cudaMalloc(&R.desc, d.size() * sizeof(ResidentMember)));
-    const int n_part = R.csize * (R.threads / 32);  // warps of a cluster, each with its part of the trace
-    const size_t per_step = (size_t)R.clusters * n_part * 2;  // doubles of one step's trace parts
-    // steps per launch: bounded so that a launch stays well below a second and the parts below 64 MB
-    const long most = std::max<long>(1, std::min<long>(4096, (8l << 20) / (long)per_step));
-    if (record) {
-        const size_t need = per_step * (size_t)std::min(most, n_steps);
-        if (R.part_cap < need) {
-            if (R.part) cudaFree(R.part);
-            R.part = nullptr;
-            R.part_cap = 0;
-            QH_CK(h, dalloc(&R.part, need));
-            R.part_cap = need;
-        }
-    }
+    const int n_part = resident_parts(R);
+    const long most = resident_steps(R);
     for (long done = 0; done < n_steps;) {
         const int len = (int)std::min(most, n_steps - done);
         int cluster = 0;
@@ -1193,24 +1214,25 @@ bool resident_ok(qhfpe *h, Prop &P)
 qhfpe_status run_steps(qhfpe *h, Prop &P, long n_steps, double *trace_dev, long stride)
 {
     cudaStream_t st = h->stream;
-    const bool resident = n_steps > 0 && resident_ok(h, P);
+    const bool record = trace_dev != nullptr;
+    bool resident = n_steps > 0 && resident_ok(h, P);
+    if (resident) {
+        qhfpe_status r = resident_prepare(h, {&P}, {h->U.data()}, record, P.res, n_steps, st, &resident);
+        if (r != QHFPE_OK) return r;
+    }
     if (!resident && !P.tq && P.m->fused && n_steps > 0) {
         qhfpe_status r = autotune(h, P);
         if (r != QHFPE_OK) return r;
     }
-    const bool record = trace_dev != nullptr;
     if (record) {
         set_sink_kernel<<<1, 1, 0, st>>>(P.sink, trace_dev, stride, 0);
         QH_CK(h, cudaGetLastError());
         if (P.mixed) QH_CK(h, launch_trace<double>(P.g, P.y0, P.g.tier0_rep_stride, P.m->mu, P.sink, 1, P.partial, st, P.m->trace_mu_q()));
         else QH_CK(h, launch_trace<double>(P.g, (const double *)P.y, P.g.rep_stride, P.m->mu, P.sink, 1, P.partial, st, P.m->trace_mu_q()));
     }
-    if (resident) {
-        qhfpe_status r = resident_tables(h, *P.m, h->U.data(), st);
-        if (r != QHFPE_OK) return r;
+    if (resident)
         return run_resident(h, {&P}, record ? std::vector<double *>{trace_dev} : std::vector<double *>{}, stride, P.res,
                             n_steps, st);
-    }
     if (n_steps > 0 && persistent_ok(h, P)) return run_persistent(h, P, n_steps, trace_dev, stride);
     if (h->timing.enabled) {
         for (long s = 0; s < n_steps; ++s) {
@@ -2640,16 +2662,19 @@ qhfpe_status qhfpe_batch_step(qhfpe_batch_t *b, long n_steps, double *const *tra
     cudaStream_t st = h0->stream;
     bool resident = n_steps > 0;
     for (qhfpe *h : b->mem) resident = resident && resident_wanted(h, *h->main);
+    const bool record = trace_out != nullptr;
+    std::vector<Prop *> props;
+    std::vector<const double *> U;
+    for (qhfpe *h : b->mem) {
+        props.push_back(h->main.get());
+        U.push_back(h->U.data());
+    }
     if (resident) {
-        if (b->res_state == 0) {
-            std::vector<const Prop *> props;
-            for (qhfpe *h : b->mem) props.push_back(h->main.get());
-            b->res_state = resident_plan(props, b->res) ? 1 : -1;
-        }
+        if (b->res_state == 0) b->res_state = resident_plan({props.begin(), props.end()}, b->res) ? 1 : -1;
         resident = b->res_state > 0;
     }
+    if (resident && (r = resident_prepare(h0, props, U, record, b->res, n_steps, st, &resident)) != QHFPE_OK) return r;
     if (!resident && !b->tq && n_steps > 0 && (r = batch_autotune(b, st)) != QHFPE_OK) return r;
-    const bool record = trace_out != nullptr;
     const long stride = n_steps + 1;
     if (record)
         for (qhfpe *h : b->mem) {
@@ -2666,13 +2691,9 @@ qhfpe_status qhfpe_batch_step(qhfpe_batch_t *b, long n_steps, double *const *tra
         }
     long done = 0;
     if (resident) {
-        std::vector<Prop *> props;
         std::vector<double *> traces;
-        for (qhfpe *h : b->mem) {
-            if ((r = resident_tables(h, *h->model, h->U.data(), st)) != QHFPE_OK) return r;
-            props.push_back(h->main.get());
-            if (record) traces.push_back(h->main->trace_buf);
-        }
+        for (Prop *P : props)
+            if (record) traces.push_back(P->trace_buf);
         if ((r = run_resident(h0, props, traces, stride, b->res, n_steps, st)) != QHFPE_OK) return r;
         done = n_steps;
     }
