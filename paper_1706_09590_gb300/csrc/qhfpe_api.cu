@@ -170,8 +170,8 @@ struct Model {
     std::vector<double> mu_host;
     ElemInfo *elems = nullptr;
     double *mu = nullptr;
-    double *tab64 = nullptr;   // D | L | R | twiddles, FP64
-    float *tab32 = nullptr;    // same in FP32
+    double *tab64 = nullptr;   // shapes without a fused kernel: D | L | R | twiddles, FP64
+    float *tab32 = nullptr;    // ... or FP32
     size_t tab_n = 0;          // entries of one of D, L, R
     double max_rate = 0.0;     // Gershgorin estimate of the generator's spectral radius
     std::vector<double> adia_host;  // adiabatic eigenvectors of U(q_i): [nq][S][S], v[j][a]
@@ -200,8 +200,9 @@ struct Model {
     float *tcN = nullptr;       // tensor-core path: FP32 tables in natural mode order (D | L | R)
     void *tcB = nullptr;        // tensor-core path: pre-swizzled bf16 hi/lo cosine and sine tiles
     bool fused = false;         // fused stage kernel available for (np, S)
-    double *ftab64 = nullptr;   // its tables (digit-reversed order, np twiddles)
+    double *ftab64 = nullptr;   // its tables (digit-reversed order, np twiddles), of the precision that runs the model
     float *ftab32 = nullptr;
+    double *tw64 = nullptr;     // the FP64 form's twiddles alone (the non-Condon dipole's transform, any precision)
     int tuned_tq = 0, tuned_form = -1;  // ground model: the tile that the first equilibration chose
     float *rtab = nullptr;      // resident propagation: D | L | R | lpp in its transform's order (built on first use)
     FusedTables<double> f64() const
@@ -222,6 +223,7 @@ struct Model {
         if (ftab64) cudaFree(ftab64);
         if (rtab) cudaFree(rtab);
         if (ftab32) cudaFree(ftab32);
+        if (tw64) cudaFree(tw64);
         if (tcN) cudaFree(tcN);
         if (tcB) cudaFree(tcB);
         if (adia) cudaFree(adia);
@@ -422,7 +424,15 @@ void build_tables(const Model &M, const double *U, std::vector<double> &out, F f
         }
 }
 
-qhfpe_status build_model(qhfpe *h, Model &M, int S, const double *U, const double *mu, int closure_override = -1)
+// |v| <= 2^62 rounded to the nearest integer, halves to even (llrint, which is a call here)
+long long nearest(double v)
+{
+    const double big = std::copysign(0x1p52, v);
+    return (long long)(std::fabs(v) < 0x1p52 ? (v + big) - big : v);
+}
+
+// mixed: the precision of the propagators that run the model; only its tables are made
+qhfpe_status build_model(qhfpe *h, Model &M, int S, const double *U, const double *mu, bool mixed, int closure_override = -1)
 {
     qhfpe_params p = h->p;
     if (closure_override >= 0) p.closure = closure_override;
@@ -587,45 +597,57 @@ qhfpe_status build_model(qhfpe *h, Model &M, int S, const double *U, const doubl
     }
     QH_CK(h, dalloc(&M.adia, M.adia_host.size()));
     QH_CK(h, cudaMemcpyAsync(M.adia, M.adia_host.data(), sizeof(double) * M.adia_host.size(), cudaMemcpyHostToDevice, st));
-    QH_CK(h, dalloc(&M.tab64, tab.size()));
-    QH_CK(h, cudaMemcpyAsync(M.tab64, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice, st));
-    std::vector<float> tab32(tab.begin(), tab.end());
-    QH_CK(h, dalloc(&M.tab32, tab32.size()));
-    QH_CK(h, cudaMemcpyAsync(M.tab32, tab32.data(), sizeof(float) * tab32.size(), cudaMemcpyHostToDevice, st));
-    if (M.fused) {
+    if (!M.fused) {
+        std::vector<float> tab32;
+        if (mixed) {
+            tab32.assign(tab.begin(), tab.end());
+            QH_CK(h, dalloc(&M.tab32, tab32.size()));
+            QH_CK(h, cudaMemcpyAsync(M.tab32, tab32.data(), sizeof(float) * tab32.size(), cudaMemcpyHostToDevice, st));
+        } else {
+            QH_CK(h, dalloc(&M.tab64, tab.size()));
+            QH_CK(h, cudaMemcpyAsync(M.tab64, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice, st));
+        }
+    } else {
         std::vector<double> ft;
         build_tables(M, U, ft, [&](int pos) { return fused_fft_frequency(p.np, pos); }, p.np, true);
-        std::vector<float> ft32(ft.begin(), ft.end());
+        if (mixed) {
+            const std::vector<float> ft32(ft.begin(), ft.end());
+            QH_CK(h, dalloc(&M.ftab32, ft32.size()));
+            QH_CK(h, cudaMemcpyAsync(M.ftab32, ft32.data(), sizeof(float) * ft32.size(), cudaMemcpyHostToDevice, st));
+            QH_CK(h, (prepare_fused<float, true>(p.np, S)));
+        }
         // the FP64 form's transforms and mixing run on integers (FusedTables): twiddles times 2^62, each row of a
         // table times 2^(62 - k) with 2^k above its largest value; the exponents k follow
+        double *tw = ft.data() + 3 * M.tab_n;
         for (int t = 0; t < 2 * p.np; ++t) {
             const long double a = 2.0L * std::acos(-1.0L) * (t / 2) / p.np;
             const long long w = std::llrint((t % 2 ? std::sin(a) : std::cos(a)) * 0x1p62L);
-            std::memcpy(&ft[3 * M.tab_n + t], &w, sizeof(w));
+            std::memcpy(&tw[t], &w, sizeof(w));
         }
-        const size_t n_rows = 3 * M.tab_n / p.np;
-        std::vector<int> kx(n_rows + n_rows % 2, 0);
-        for (size_t r = 0; r < n_rows; ++r) {
-            double *row = ft.data() + r * p.np, big = 0.0;
-            for (int t = 0; t < p.np; ++t) big = std::max(big, std::fabs(row[t]));
-            int k = -4096;  // a row of zeros (EXP_NO_TABLE): below every other term
-            if (big > 0.0) std::frexp(big, &k);
-            kx[r] = k;
-            const bool plain = std::abs(k) < 900;  // 2^(62 - k) is a normal double: the product is exact
-            const double scale = plain ? std::ldexp(1.0, 62 - k) : 0.0;
-            for (int t = 0; t < p.np; ++t) {
-                const long long c = big > 0.0 ? std::llrint(plain ? row[t] * scale : std::ldexp(row[t], 62 - k)) : 0;
-                std::memcpy(row + t, &c, sizeof(c));
+        QH_CK(h, dalloc(&M.tw64, 2 * p.np));
+        QH_CK(h, cudaMemcpyAsync(M.tw64, tw, sizeof(double) * 2 * p.np, cudaMemcpyHostToDevice, st));
+        if (!mixed) {
+            const size_t n_rows = 3 * M.tab_n / p.np;
+            std::vector<int> kx(n_rows + n_rows % 2, 0);
+            for (size_t r = 0; r < n_rows; ++r) {
+                double *row = ft.data() + r * p.np, big = 0.0;
+                for (int t = 0; t < p.np; ++t) big = std::max(big, std::fabs(row[t]));
+                int k = -4096;  // a row of zeros (EXP_NO_TABLE): below every other term
+                if (big > 0.0) std::frexp(big, &k);
+                kx[r] = k;
+                const bool plain = std::abs(k) < 900;  // 2^(62 - k) is a normal double: the product is exact
+                const double scale = plain ? std::ldexp(1.0, 62 - k) : 0.0;
+                for (int t = 0; t < p.np; ++t) {
+                    const long long c = big > 0.0 ? nearest(plain ? row[t] * scale : std::ldexp(row[t], 62 - k)) : 0;
+                    std::memcpy(row + t, &c, sizeof(c));
+                }
             }
+            const size_t ft_n = 3 * M.tab_n + 3 * p.np;
+            QH_CK(h, dalloc(&M.ftab64, ft_n + kx.size() / 2));
+            QH_CK(h, cudaMemcpyAsync(M.ftab64, ft.data(), sizeof(double) * ft_n, cudaMemcpyHostToDevice, st));
+            QH_CK(h, cudaMemcpyAsync(M.ftab64 + ft_n, kx.data(), sizeof(int) * kx.size(), cudaMemcpyHostToDevice, st));
+            QH_CK(h, (prepare_fused<double, false>(p.np, S)));
         }
-        const size_t ft_n = 3 * M.tab_n + 3 * p.np;
-        QH_CK(h, dalloc(&M.ftab64, ft_n + kx.size() / 2));
-        QH_CK(h, cudaMemcpyAsync(M.ftab64, ft.data(), sizeof(double) * ft_n, cudaMemcpyHostToDevice, st));
-        QH_CK(h, cudaMemcpyAsync(M.ftab64 + ft_n, kx.data(), sizeof(int) * kx.size(), cudaMemcpyHostToDevice, st));
-        QH_CK(h, dalloc(&M.ftab32, ft32.size()));
-        QH_CK(h, cudaMemcpyAsync(M.ftab32, ft32.data(), sizeof(float) * ft32.size(), cudaMemcpyHostToDevice, st));
-        QH_CK(h, (prepare_fused<float, true>(p.np, S)));
-        QH_CK(h, (prepare_fused<double, false>(p.np, S)));
     }
     if (p.precision == QHFPE_MIXED_BF16X3 && tc_supported(p.np, S)) {
         std::vector<double> nt;
@@ -1346,11 +1368,11 @@ qhfpe_status apply_dipole_prop(qhfpe *h, Prop &P, int side, const int *reps_dev,
             // FP32 pass over every element, then the FP64 zeroth tier (which also rewrites its FP32 copy)
             QH_CK(h, launch_dipole_fft<float>(P.g, M.dip32, M.dip32 + tn, M.ftab32 + 3 * tn, (float *)P.y, P.g.rep_stride,
                                               M.n_elem, reps_dev, n, side, scale, nullptr, 0, h->stream));
-            QH_CK(h, launch_dipole_fft<double>(P.g, M.dip64, M.dip64 + tn, M.ftab64 + 3 * tn, P.y0,
+            QH_CK(h, launch_dipole_fft<double>(P.g, M.dip64, M.dip64 + tn, M.tw64, P.y0,
                                                P.g.tier0_rep_stride, 1, reps_dev, n, side, scale, (float *)P.y,
                                                P.g.rep_stride, h->stream));
         } else {
-            QH_CK(h, launch_dipole_fft<double>(P.g, M.dip64, M.dip64 + tn, M.ftab64 + 3 * tn, (double *)P.y,
+            QH_CK(h, launch_dipole_fft<double>(P.g, M.dip64, M.dip64 + tn, M.tw64, (double *)P.y,
                                                P.g.rep_stride, M.n_elem, reps_dev, n, side, scale, nullptr, 0,
                                                h->stream));
         }
@@ -1500,7 +1522,7 @@ qhfpe_status qhfpe_create(const qhfpe_params *params, void *stream, qhfpe_t **ou
         }
     }
     h->model.reset(new Model());
-    qhfpe_status r = build_model(h.get(), *h->model, S, h->U.data(), h->mu.data());
+    qhfpe_status r = build_model(h.get(), *h->model, S, h->U.data(), h->mu.data(), p.precision != QHFPE_FP64);
     if (r != QHFPE_OK) {
         create_err = h->err;
         return r;
@@ -1951,7 +1973,7 @@ qhfpe_status equilibrium_start(qhfpe_t *h, std::unique_ptr<Prop> &GP)
         h->ground.reset(new Model());
         // the state-input closure's network is for n_states pairs: the ground problem is closed by the
         // Eq. (GMFP) terminator
-        r = build_model(h, *h->ground, 1, U00.data(), &zero,
+        r = build_model(h, *h->ground, 1, U00.data(), &zero, false,
                         p.closure == QHFPE_LEARNED_STATE ? (int)QHFPE_TERMINATOR : -1);
         if (r != QHFPE_OK) return r;
     }
