@@ -8,7 +8,7 @@
 // sums are exact, and twiddle products keep the upper 64 of 128 bits.  An FFT mixes all points of a row, so
 // its rounding error is relative to the row's norm in either arithmetic; with 58 to 60 bits below the
 // largest input and a binary point that follows the growth of the sums, that error is smaller than the FP64
-// butterflies' (tests/test_fixed_fft.py bounds it against extended precision).
+// butterflies' (forward 4e-17 to 1.3e-16 against 8e-17 to 2.1e-16 of the norm, tests/test_fixed_fft_fp64.py).
 //
 // Magnitudes (complex): a radix-16 pass takes inputs below 2^60 and scales by 1/4 between its two layers
 // of length-4 transforms (outputs below 2^62); a radix-8 pass takes inputs below 2^59; a twiddle product
