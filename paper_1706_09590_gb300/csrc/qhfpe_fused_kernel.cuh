@@ -789,7 +789,7 @@ template <int VEC, typename T> __device__ __forceinline__ void with_neighbours(c
 //            four steps of 96 x 128 at depth 8 took 9.26 ms, this way 8.11.)
 //   tiers    G = sum of the neighbours' rows, weighted, in FP64 (one instruction per value and neighbour, on a
 //            pipe that has room for them; in integers the conversions alone took twenty); its row is brought
-//            to the largest exponent, 57 bits below it, and the p difference (weights 1, 8) is exact.
+//            to the largest exponent, 58 bits below it, and the p difference (weights 1, 8) is exact.
 // Quantising at 2^-54 to 2^-62 of the largest term is below the rounding of the FP64 sums, whose partial sums of
 // up to 100 times the values round at 2^-53.
 // Rows whose differences or potential term are near the ends of the range of doubles (exp_plain) have their q differences
@@ -804,7 +804,7 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
     constexpr int S2 = S * S;
     constexpr int VEC = NP / 32;              // a warp holds a p row
     constexpr int RG = 4;                     // q rows per unit, at most
-    constexpr int BITS = 57;                  // of G below its row's largest value: 18 x 2^57 stays below 2^62
+    constexpr int BITS = 58;                  // of G below its row's largest value: 18 x 2^58 stays below 2^63
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t blk = g.blk;
     const int nq = g.nq;
