@@ -1022,7 +1022,6 @@ qhfpe_status persistent_desc(qhfpe *h, Prop &P)
     x.elems = M.elems;
     if constexpr (sizeof(T) == 4) x.tab = M.f32();
     else x.tab = M.f64();
-    x.sc[0] = stage_scalars<T>(P.g, 0.0);
     for (int k = 1; k <= 4; ++k) x.sc[k] = stage_scalars<T>(P.g, P.dt / k);
     x.dt = P.dt;
     x.y = (T *)P.y;
@@ -2533,7 +2532,6 @@ qhfpe_status batch_upload(qhfpe_batch *b, int tq)
         x.elems = M.elems;
         if constexpr (sizeof(T) == 4) x.tab = M.f32();
         else x.tab = M.f64();
-        x.sc[0] = stage_scalars<T>(P.g, 0.0);
         for (int k = 1; k <= 4; ++k) x.sc[k] = stage_scalars<T>(P.g, P.dt / k);
         x.dt = P.dt;
         x.y = (T *)P.y;
@@ -2565,8 +2563,8 @@ qhfpe_status batch_launch(qhfpe_batch *b, int k, cudaStream_t st)
     return QHFPE_OK;
 }
 
-// the batch's tile height: every candidate evaluates every member's right-hand side (into its second
-// stage buffer, which holds no data between steps) a few times, timed with CUDA events
+// the batch's tile height: every candidate runs the first three stages of a step, into the stage buffers (which
+// hold no data between steps), timed with CUDA events
 qhfpe_status batch_autotune(qhfpe_batch *b, cudaStream_t st)
 {
     qhfpe *h0 = b->mem[0];
@@ -2590,11 +2588,10 @@ qhfpe_status batch_autotune(qhfpe_batch *b, cudaStream_t st)
         if (r != QHFPE_OK) return r;
         b->tq = tq;
         float ms = 0.f;
-        for (int rep = 0; rep < 4; ++rep) {
-            if (rep == 1) QH_CK(h0, cudaEventRecord(e0, st));
-            r = batch_launch(b, 0, st);
-            if (r != QHFPE_OK) return r;
-        }
+        if ((r = batch_launch(b, 4, st)) != QHFPE_OK) return r;  // warm-up
+        QH_CK(h0, cudaEventRecord(e0, st));
+        for (int k = 4; k >= 2; --k)
+            if ((r = batch_launch(b, k, st)) != QHFPE_OK) return r;
         QH_CK(h0, cudaEventRecord(e1, st));
         QH_CK(h0, cudaEventSynchronize(e1));
         QH_CK(h0, cudaEventElapsedTime(&ms, e0, e1));

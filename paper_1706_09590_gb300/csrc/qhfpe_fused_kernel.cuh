@@ -1170,12 +1170,11 @@ __device__ __forceinline__ void row_wide(const GridInfo &g, const StageScalars<f
 // grid, surfaces, bath, hierarchy depth, closure, dt and replica count, and share NP, S and the
 // precision).  Blocks are numbered member by member; a block finds its member (first block numbers
 // ascending), copies the member's description into shared memory and does that member's block of stage
-// k = 4..1 of the Horner form (k = 0: the right-hand side alone into the second stage buffer, for the
-// autotuner).  The other arguments are then taken from the member.
+// k = 4..1 of the Horner form.  The other arguments are then taken from the member.
 // The block `bid` of a fused stage launch (see fused_stage_kernel below); also called in a loop by the
 // persistent kernel (a barrier must separate two calls of one block: shared memory is reused).
 // NL: the terms of the nonlinear coupling (GridInfo::c2 != 0) are compiled in; NL = false requires
-// c2 = 0 (the linear coupling of every workload but the NEXT-3b one keeps their registers free).
+// c2 = 0 (the linear coupling keeps their registers free).
 template <typename T, int NP, int S, bool MIXED, bool MULTI, bool NL>
 __device__ __forceinline__ void
 fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<T> tab, StageScalars<T> sc,
@@ -1206,13 +1205,13 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
         elems = M.elems;
         tab = M.tab;
         sc = M.sc[k];
-        v_in = k == 4 || k == 0 ? M.y : (k == 3 ? M.vA : (k == 2 ? M.vB : M.vA));
+        v_in = k == 4 ? M.y : (k == 2 ? M.vB : M.vA);
         y = M.y;
         y0 = M.y0;
-        v_out = k == 0 ? M.vB : (k == 1 ? M.y : (k == 4 ? M.vA : (k == 3 ? M.vB : M.vA)));
+        v_out = k == 1 ? M.y : (k == 3 ? M.vB : M.vA);
         y0_out = k == 1 ? M.y0 : nullptr;
-        h = k == 0 ? 0.0 : M.dt / k;
-        mode = k == 0 ? 0 : (k == 1 ? 2 : 1);
+        h = M.dt / k;
+        mode = k == 1 ? 2 : 1;
         terms = QHFPE_TERM_ALL;
         rep0 = 0;
         n_rep = M.g.n_rep;

@@ -102,7 +102,7 @@ struct MultiMember {
     GridInfo g;
     const ElemInfo *elems;
     FusedTables<T> tab;
-    StageScalars<T> sc[5];  // [k]: stage k = 1..4 (h = dt / k); [0]: the right-hand side alone (h = 0)
+    StageScalars<T> sc[5];  // [k]: stage k = 1..4 (h = dt / k)
     double dt;
     T *y, *vA, *vB;
     double *y0;             // FP64 zeroth tier (mixed form), else nullptr
