@@ -2500,9 +2500,6 @@ struct qhfpe_batch {
     long blocks = 0;
     void *desc = nullptr;  // device MultiMember<float or double>[n]
     cudaGraphExec_t graphs[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [chunk][trace]
-    void *pdesc = nullptr;      // persistent propagation: this propagator as a one-member batch
-    int pdesc_tq = 0;           // its tile height
-    unsigned *pbar = nullptr;   // barrier words (count, generation) and the give-up flag
     int res_state = 0;          // resident propagation: 0 not yet decided, 1 taken, -1 not
     ResidentPlan res;
     ~qhfpe_batch()

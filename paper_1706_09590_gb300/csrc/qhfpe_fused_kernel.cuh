@@ -1019,8 +1019,7 @@ template <int NP, bool MIXED>
 __device__ __forceinline__ void row_wide(const GridInfo &g, const StageScalars<float> &sc, const float *__restrict__ v_in,
                                          const float *y, const double *y0, float *v_out, double *y0_out, double h, int mode,
                                          bool tier0, size_t o, size_t o0, int i, const float *pcol, bool interior,
-                                         const long long *nb_off, const float *nb_wg, const float *nb_wa, int n_up,
-                                         int n_d0, int n_nb, bool term, const float2 *xp)
+                                         const long long *nb_off, const float *nb_wg, const float *nb_wa, int n_d0, int n_nb, bool term, const float2 *xp)
 {
     constexpr int VEC = NP / 32, NB = 3;
     const size_t blk = g.blk;
@@ -1394,7 +1393,7 @@ fused_stage_body(unsigned bid, GridInfo g, const ElemInfo *__restrict__ elems, F
             if (uni_warp && fold && terms == QHFPE_TERM_ALL) {
                 row_wide<NP, MIXED>(g, sc, v_in, y, y0, v_out, y0_out, h, mode, MIXED && e == 0, o,
                                     (size_t)rep * g.tier0_rep_stride + (size_t)pr * 2 * blk + (size_t)i * NP + l0, i, pcol,
-                                    interior, nb_off, nb_wg, nb_wa, n_up, n_d0, n_nb, term,
+                                    interior, nb_off, nb_wg, nb_wa, n_d0, n_nb, term,
                                     X + pad16((r * S2 + pr) * NP + l0));
                 continue;
             }
