@@ -973,7 +973,7 @@ qhfpe_status autotune(qhfpe *h, Prop &P)
         const int tiles = (P.g.nq + c - 1) / c, level = (P.g.nq + tiles - 1) / tiles;  // as many tiles, of one height
         for (int tq : {level, c}) {
             // the FP64 form works on groups of four q rows of the grid: multiples of four as they are, too (97 rows of
-            // one state, np 128: tiles of 14 rows 23.1 ms for an equilibration, of 16 rows 22.5)
+            // one state, np 128: an equilibration is up to 2 % faster with tiles of 16 rows than of 14)
             if (timed[tq] || (tq != level && (P.mixed || tq % 4 != 0))) continue;
             timed[tq] = true;
             qhfpe_status r = time_one(0, tq, &ms);

@@ -36,8 +36,9 @@ constexpr int EXP_BAD = 16000;
 // ... of a row of zeros, and the exponent of a table row of zeros: sums with one of those are below EXP_ZERO (others are
 // above -1300), and the values zero
 constexpr int EXP_NONE = -6000, EXP_NO_TABLE = -4096, EXP_ZERO = -1500;
-// exponents of doubles outside of these (values below 2^-895, from 2^1007) take the functions for any value
-constexpr int EXP_SMALL = 128, EXP_BIG = 2030;
+// exponents of doubles outside of these (values below 2^-895, from 2^927) take the functions for any value; between
+// them rates from 2^-60 to 2^90 leave normal numbers
+constexpr int EXP_SMALL = 128, EXP_BIG = 1950;
 QH_HD bool exp_far(int M) { return (unsigned)(M - EXP_SMALL) >= (unsigned)(EXP_BIG - EXP_SMALL) && M >= EXP_ZERO; }
 QH_HD bool exp_plain(int E) { return (unsigned)(E - EXP_SMALL) < (unsigned)(EXP_BIG - EXP_SMALL); }
 

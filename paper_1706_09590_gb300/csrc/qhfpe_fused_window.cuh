@@ -46,8 +46,8 @@ template <int NP, int S, int TQ, bool PG> constexpr size_t win_smem()
 }
 
 // PG: the potential term is read from Pg (the tensor-core form); phase A is left out, and the p-diagonal
-// bath terms are applied to the centre row instead of in r-space.  On 96 x 128 at depth 8 the tensor-core form's
-// step went from 0.699 to 0.680 ms (general kernel to this one).
+// bath terms are applied to the centre row instead of in r-space.  Twelve steps of the tensor-core
+// form on 96 x 128 at depth 8: 8.40 -> 8.25 to 8.35 ms (general kernel to this one).
 template <int NP, int S, bool MIXED, bool PG>
 __global__ void __launch_bounds__(FTHREADS, WIN_BLOCKS)
 fused_window_kernel(GridInfo g, const ElemInfo *__restrict__ elems, FusedTables<float> tab, StageScalars<float> sc,

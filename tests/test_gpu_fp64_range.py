@@ -110,3 +110,19 @@ def test_an_infinity_reaches_what_it_reaches(name):
     # (not bit for bit: where a column's values are far apart its neighbours' sums are taken at another unit)
     assert np.linalg.norm(got[~hit] - clean[~hit]) < TOL * np.linalg.norm(clean[~hit])
     assert not np.isfinite(got[0, 1, 0, 4]).any() and not np.isfinite(got[0, 1, 0, [4 + d for d in reach], 9]).any()
+
+
+@pytest.mark.parametrize("k", [-850, 900, 990, 1006])
+def test_large_rates(k):
+    """Fast q differences (p / 60 dq up to 2^20) of values near the ends: finite results, infinities where they overflow."""
+    m = qi.harmonic_two_state(nq=9, n_p=32, qr=(-1e-5, 1e-5), pr=(-128.0, 128.0), depth=1, eta=0.0)
+    W = qi.random_state(m, seed=94)
+    h = k // 2
+    P = _P(m)
+    ref = _rhs(P, W)
+    got = _rhs(P, W * 2.0 ** h * 2.0 ** (k - h))
+    P.close()
+    back = (got * 2.0 ** -h) * 2.0 ** (h - k)
+    fits = np.abs(ref) < 2.0 ** min(1022 - k, 1000)
+    assert (np.abs(back - ref)[fits] <= 16 * TOL * np.broadcast_to(_rows(ref)[..., None], ref.shape)[fits]).all()
+    assert not np.isfinite(got[~(np.abs(ref) < 2.0 ** min(1025 - k, 1000))]).any()
