@@ -527,6 +527,7 @@ qhfpe_status build_model(qhfpe *h, Model &M, int S, const double *U, const doubl
     g.log2np = M.log2np;
     g.n_elem = M.n_elem;
     g.n_rep = 0;
+    g.q_group = 4;
     g.periodic_q = p.periodic_q;
     g.q_min = p.q_min;
     g.p_min = p.p_min;
@@ -672,6 +673,7 @@ qhfpe_status make_prop(qhfpe *h, Model *M, int n_rep, bool mixed, double dt, std
     P->m = M;
     P->g = M->g;
     P->g.n_rep = n_rep;
+    P->g.q_group = fused_q_group(P->g);
     P->mixed = mixed;
     P->tc = mixed && M->tcB != nullptr;
     P->dt = dt;

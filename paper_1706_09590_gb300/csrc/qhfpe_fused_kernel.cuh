@@ -470,9 +470,6 @@ template <int NP> struct FixedRows {
     }
 };
 
-// (a function of its own: few rows need it)
-template <int B> __device__ __noinline__ long long far_fixed(double v, int E) { return qhfx::to_fixed_any<B>(v, E); }
-
 // rows * S2 p-rows of the tile into X as integers below 2^bits of their row's exponent
 template <int NP, int S2>
 __device__ __forceinline__ void fill_fixed(double2 *X, const double *__restrict__ v, size_t blk, int i0, int rows)
@@ -511,7 +508,7 @@ __device__ __forceinline__ void fill_fixed(double2 *X, const double *__restrict_
                 for (int q = 0; q < LV; ++q) x[q] = I2{0, 0};
             } else {
 #pragma unroll
-                for (int q = 0; q < LV; ++q) x[q] = I2{far_fixed<B>(re[q], E), far_fixed<B>(im[q], E)};
+                for (int q = 0; q < LV; ++q) x[q] = I2{to_fixed_any<B>(re[q], E), to_fixed_any<B>(im[q], E)};
             }
             if (l == 0) F::exp_slot(X, rp, F::FWD_EXP) = (short)(E < 2047 ? E : EXP_BAD);
         }
@@ -736,7 +733,7 @@ __device__ __forceinline__ int upwind_weight(bool neg, int t)
 }
 
 // A value's q difference times pk, in FP64, and its potential term pot 2^K: the column V, window rows from ii on
-__device__ __noinline__ double far_value(const double *V, int np, int ii, int nq, int periodic, bool neg, double pk,
+__device__ __forceinline__ double far_value(const double *V, int np, int ii, int nq, int periodic, bool neg, double pk,
                                          long long pot, int K)
 {
     double kin = 0.0;
@@ -783,10 +780,10 @@ template <int VEC, typename T> __device__ __forceinline__ void with_neighbours(c
 //   kinetic  the q differences have small integer weights (sum of sizes 130).  A warp takes four rows of one
 //            pair; for each of its p columns the nine rows read are brought to the column's largest exponent
 //            (62 bits below it) once, and the four sums of six are exact.  Where the rows' own exponents are
-//            more than eight apart each of the four takes its own.  The four are rows 4 n .. 4 n + 3 of the grid:
-//            a unit that holds only some of them, at the edge of a tile or in a small one, reads all nine rows
-//            all the same, so that results don't depend on the tile.  (With an exponent for each row everywhere
-//            four steps of 96 x 128 at depth 8 took 9.26 ms, this way 8.1 to 8.2.)
+//            more than eight apart each of the four takes its own.  The four are rows 4 n .. 4 n + 3 of the grid
+//            (or three, np >= 128: GridInfo::q_group): a unit that holds only some of them, at the edge of a tile or in a small one,
+//            reads all nine rows all the same, so that results don't depend on the tile.  (With an exponent for each row
+//            everywhere four steps of 96 x 128 at depth 8 took 9.26 ms, this way 8.1 to 8.2.)
 //   tiers    G = sum of the neighbours' rows, weighted, in FP64 (one instruction per value and neighbour, on a
 //            pipe that has room for them; in integers the conversions alone took twenty); its row is brought
 //            to the largest exponent, 58 bits below it, and the p difference (weights 1, 8) is exact.
@@ -815,15 +812,16 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
     for (int t = 0; t < 6; ++t) ck[t] = upwind_weight(neg, t);
     const int first = neg ? -2 : -3;
     const double bad = bitsd(0x7ff8000000000000ull);
-    int rg = min(RG, (rows * S2 + FTHREADS / 32 - 1) / (FTHREADS / 32));  // fewer where warps would idle
-    rg = rg == 3 ? RG : rg;
+    const int gr = NP >= 128 ? g.q_group : RG;
+    int rg = min(gr, (rows * S2 + FTHREADS / 32 - 1) / (FTHREADS / 32));  // fewer where warps would idle
+    if (2 * rg > gr) rg = gr;
     const int u0 = i0 / rg, n_u = (i0 + rows - 1) / rg - u0 + 1;  // units of rg rows, aligned on the grid
 #pragma unroll 1
     for (int u = warp; u < n_u * S2; u += FTHREADS / 32) {
         const int pr = u % S2, us = (u0 + u / S2) * rg;
         const int ia = max(us, i0), r0 = ia - i0;
         const int nr = min(us + rg, i0 + rows) - ia;
-        const int gs = ia & ~(RG - 1), k0 = ia - gs;  // the group of RG grid rows that the unit's are among
+        const int gs = NP < 128 ? ia & ~(RG - 1) : ia - ia % gr, k0 = ia - gs;  // the group of grid rows that the unit's are among
         const size_t poff = ebase + (size_t)pr * 2 * blk;
         // the unit's rows in the group, by the exponent of their potential term
         unsigned near = ((1u << nr) - 1) << k0, far = 0;
@@ -883,7 +881,7 @@ rows_fixed(const GridInfo &g, const StageScalars<double> &sc, const double *__re
 #pragma unroll
                 for (int r = 0; r < RG; ++r) {
                     const int er = max(max(max(ex[r], ex[r + 1]), max(ex[r + 2], ex[r + 3])), max(ex[r + 4], ex[r + 5]));
-                    if (gs + r < nq) least = min(least, er);
+                    if (r < gr && gs + r < nq) least = min(least, er);
                 }
                 unsigned odd = far;  // rows left to FP64
                 bool zero = false;  // nothing but zeros in the window

@@ -42,6 +42,7 @@ struct GridInfo {
     int S, nq, np, log2np;
     int n_elem, n_rep;
     int periodic_q;
+    int q_group;       // FP64 form: q rows that share an exponent in their differences, aligned on the grid (fused_q_group)
     double q_min, p_min, dq, dp;
     double cdelta;     // delta-term coefficient
     double term_r0, term_c0;  // terminator coefficients (r_0, c_0)
@@ -158,6 +159,7 @@ cudaError_t launch_fused(const GridInfo &g, const ElemInfo *elems, const FusedTa
 // QHFPE_FUSED_WINDOW=0; its q rows per block.
 bool fused_window_applies(const GridInfo &g, int terms);
 int fused_window_rows(int S);
+int fused_q_group(const GridInfo &g);  // GridInfo::q_group of a propagator
 int fused_max_rows(int np, int S, int elem_bytes);
 template <typename T>
 StageScalars<T> stage_scalars(const GridInfo &g, double h);

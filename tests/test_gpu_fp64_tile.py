@@ -13,7 +13,10 @@ def _models():
             "two_32": qi.harmonic_two_state(nq=18, n_p=32, depth=3),
             "periodic_64": qi.harmonic_two_state(nq=19, n_p=64, depth=2, periodic_q=1),
             "three_64": qi.three_state(nq=13, n_p=64, depth=1, n_matsubara=1),
-            "one_256": qi.single_state(lambda q: 0.5 * q * q, nq=11, n_p=256, pr=(-16.0, 16.0), depth=2, dt=1e-3)}
+            "one_256": qi.single_state(lambda q: 0.5 * q * q, nq=11, n_p=256, pr=(-16.0, 16.0), depth=2, dt=1e-3),
+            # groups of three rows: between two and three rows of elements for each block of a wave
+            "one_128_threes": qi.single_state(lambda q: 0.5 * q * q, nq=101, n_p=128, pr=(-16.0, 16.0), depth=14, dt=1e-4),
+            "two_128_threes": qi.photoisomerization_two_state(nq=62, n_p=128, depth=3)}
 
 
 @pytest.mark.parametrize("name", list(_models()))
