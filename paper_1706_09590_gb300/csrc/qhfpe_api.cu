@@ -928,11 +928,13 @@ qhfpe_status autotune(qhfpe *h, Prop &P)
     float best = 1e30f, ms = 0.f;
     // stages of every replica into vB with the given form and tile, with a base read as in a step (vA, whatever it
     // holds, times one plus nothing: without it the general form looked 4 % faster than it is in steps of 96 x 128
-    // models): one to warm up, one timed, and two more unless that one was far behind the best so far; *ms for three
+    // models): one to warm up, one timed, and more unless that one was far behind the best so far, also when timed again (it
+    // may have been held up); *ms for three.  Short stages run eight in a row: only there the next launch's blocks
+    // start while one drains, as in a step (96 x 64, two states, depth 5: single launches favoured tiles of two rows, 85
+    // us a step, over one, 68)
     auto time_one = [&](int form, int tq, float *ms) -> qhfpe_status {
-        *ms = 0.f;
-        for (int n : {1, 2}) {
-            for (int rep = n - 2; rep < n; ++rep) {  // (n = 1: launch -1 is the warm-up)
+        auto timed = [&](int warm, int n, float *t) -> qhfpe_status {
+            for (int rep = -warm; rep < n; ++rep) {
                 if (rep == 0) QH_CK(h, cudaEventRecord(a, st));
                 cudaError_t e;
                 if (P.mixed)
@@ -945,16 +947,23 @@ qhfpe_status autotune(qhfpe *h, Prop &P)
                                                     st, nullptr, tq, form);
                 QH_CK(h, e);
             }
-            float t = 0.f;
             QH_CK(h, cudaEventRecord(b, st));
             QH_CK(h, cudaEventSynchronize(b));
-            QH_CK(h, cudaEventElapsedTime(&t, a, b));
-            *ms += t;
-            if (n == 1 && 3.f * t > 1.25f * best) {
-                *ms = 3.f * t;
-                break;
-            }
+            QH_CK(h, cudaEventElapsedTime(t, a, b));
+            return QHFPE_OK;
+        };
+        float one = 0.f, t = 0.f;
+        qhfpe_status r = timed(1, 1, &one);
+        if (r == QHFPE_OK && 3.f * one > 1.25f * best) {
+            r = timed(1, 1, &t);
+            one = std::min(one, t);
         }
+        if (r != QHFPE_OK) return r;
+        *ms = 3.f * one;
+        if (*ms > 1.25f * best) return QHFPE_OK;
+        const int n = one < 0.05f ? 8 : 2;
+        if ((r = timed(0, n, &t)) != QHFPE_OK) return r;
+        *ms = n > 2 ? 3.f * t / n : std::min(*ms, 1.5f * t);
         return QHFPE_OK;
     };
     int best_tq = 1, best_form = 0;

@@ -117,8 +117,8 @@ bool window_enabled()
 
 // Rows of the groups that share an exponent in the q differences of the FP64 form: four, but three where one wave of
 // blocks holds the stage in tiles of three rows and not of two, which are then the fastest and would lie across two
-// groups of four as often as not.  us a step with four / three: 96 x 128, two states, depth 12 256 / 210, 80 x 128 at three
-// modes, depth 3 278 / 227, three states on 64 x 128, depth 3 549 / 505.  (np 32 and 64: always four; the choice alone cost 2 to
+// groups of four as often as not.  us a step with four / three: 96 x 128, two states, depth 12 256 / 212, 80 x 128 at three
+// modes, depth 3 278 / 229, three states on 64 x 128, depth 3 549 / 517.  (np 32 and 64: always four; the choice alone cost 2 to
 // 4 % of their short stages.)  A rule of shape, not of the tile, so that results don't
 // depend on what a timing picked.
 int fused_q_group(const GridInfo &g)

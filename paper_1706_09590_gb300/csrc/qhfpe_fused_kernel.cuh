@@ -783,7 +783,7 @@ template <int VEC, typename T> __device__ __forceinline__ void with_neighbours(c
 //            more than eight apart each of the four takes its own.  The four are rows 4 n .. 4 n + 3 of the grid
 //            (or three, np >= 128: GridInfo::q_group): a unit that holds only some of them, at the edge of a tile or in a small one,
 //            reads all nine rows all the same, so that results don't depend on the tile.  (With an exponent for each row
-//            everywhere four steps of 96 x 128 at depth 8 took 9.26 ms, this way 8.1 to 8.2.)
+//            everywhere four steps of 96 x 128 at depth 8 took 9.26 ms where this way they took 8.1.)
 //   tiers    G = sum of the neighbours' rows, weighted, in FP64 (one instruction per value and neighbour, on a
 //            pipe that has room for them; in integers the conversions alone took twenty); its row is brought
 //            to the largest exponent, 58 bits below it, and the p difference (weights 1, 8) is exact.
